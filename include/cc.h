@@ -453,21 +453,22 @@ cc_status cc_set_launch_shape(cc_mesh* mesh, int32_t couple_threads, int32_t gat
 
 /* Selects between equivalent kernel variants of the sweep (no counterpart in
  * the paper; both settings compute Eq. 9-12 on the same data):
- *   rows_from_positions  1: the mixed path's stable Neo-Hookean float32 block
- *                        rows are formed per row from the positions (no
- *                        per-tet Hessian store); 0: per-tet Hessian store +
- *                        gather.  Fixed Corotational and the float64 path
- *                        always use the store.
+ *   rows_from_positions  1: stable Neo-Hookean gradients and block rows are
+ *                        formed per row from the positions (no per-tet Hessian
+ *                        store), in both precisions; 0: per-tet Hessian store +
+ *                        gather.  Fixed Corotational meshes, and meshes with a
+ *                        vertex of more than 255 neighbours or more tets than
+ *                        a CTA's shared memory holds, always use the store.
  *   fused_condense       1: the coupling kernel condenses its vertices itself
  *                        (the last CTA of every 32 list entries runs the
  *                        float64 3x3 solves of the group, one vertex per
  *                        lane); 0: a separate condensation launch.  The
  *                        one-warp coupling shape always launches it apart.
  * 1 sets, 0 clears, -1 keeps a switch; anything else is CC_ERR_INVALID_ARG.
- * Defaults: both 0 (measured fastest on the 32^3 cube); cc_autotune tries
- * every applicable combination.  The fused and separate
- * condensations give identical results; the two row builds agree within
- * float32 rounding. */
+ * Defaults (measured fastest): rows_from_positions 1, fused_condense 0;
+ * cc_autotune tries every applicable combination.  The fused and separate
+ * condensations give identical results; the two row builds agree within the
+ * rounding of the path's precision. */
 cc_status cc_set_sweep_variant(cc_mesh* mesh, int32_t rows_from_positions, int32_t fused_condense);
 
 /* ======================================================================

@@ -63,17 +63,19 @@ void ensure_state(Mesh& m, cc_precision p) {
     CCG_CUDA(cudaMemsetAsync(m.d_grp_cnt.p, 0, m.d_grp_cnt.count * sizeof(int32_t), s));
   }
   if (p == CC_PREC_FP64) {
-    if (!m.f64.gcon.p) {
+    // the per-tet store exists only where the rows are gathered from it
+    if (!rows_from_positions(m) && !m.f64.hten.p) {
       m.f64.gcon.alloc(3 * ne);
       m.f64.hten.alloc(kTetStore * (size_t)m.T);
+    }
+    if (!m.f64.g.p) {
       m.f64.g.alloc(3 * m.n);
       m.f64.bsr.alloc(12 * m.nnz_up);
       m.f64.cpl.alloc(32 * m.n_free);
       CCG_CUDA(cudaMemsetAsync(m.f64.g.p, 0, 3 * m.n * sizeof(double), s));
     }
   } else {
-    if (!m.mx.gcon.p) {
-      m.mx.gcon.alloc(3 * ne);
+    if (!m.mx.g_hi.p) {
       m.mx.g_hi.alloc(3 * m.n);
       m.mx.g_lo.alloc(3 * m.n);
       m.mx.bsr.alloc(12 * m.nnz_up);
@@ -87,8 +89,15 @@ void ensure_state(Mesh& m, cc_precision p) {
       CCG_CUDA(cudaMemsetAsync(m.mx.xt_hi.p, 0, m.n * sizeof(float4), s));
       CCG_CUDA(cudaMemsetAsync(m.mx.xt_lo.p, 0, m.n * sizeof(float4), s));
     }
-    // the per-tet Hessian store exists only for the gather path
-    if (!rows_from_positions(m) && !m.mx.hten.p) m.mx.hten.alloc(kTetStore * (size_t)m.T);
+    if (rows_from_positions(m)) {
+      if (!m.mx.rec.p) {
+        m.mx.rec.alloc(m.T);
+        CCG_CUDA(cudaMemsetAsync(m.mx.rec.p, 0, m.T * sizeof(float4), s));
+      }
+    } else if (!m.mx.hten.p) {
+      m.mx.gcon.alloc(3 * ne);
+      m.mx.hten.alloc(kTetStore * (size_t)m.T);
+    }
   }
 }
 
@@ -156,17 +165,25 @@ double elastic_weight(const Mesh& m) { return m.h > 0.0 ? m.h * m.h : 1.0; }
 // Re-evaluates the per-tet derivatives for a tet list and re-gathers g, H.
 void refresh(Mesh& m, cc_precision p, const double* x, const double* xt, const int32_t* list, int64_t count) {
   cudaStream_t s = m.stream;
-  int e0 = prof_event(m);
-  if (p == CC_PREC_FP64)
-    launch_tet_grad_f64(m, x, list, count, elastic_weight(m), s);
-  else
-    launch_tet_grad_mixed(m, list, count, elastic_weight(m), s);
-  prof_close(m, P_TET, e0, count > 0 ? 1 : 0);
+  const bool store = !rows_from_positions(m), mixed = p == CC_PREC_MIXED;
+  int e0;
+  if (store || mixed) {  // float64 rows from the positions need no per-tet pass
+    e0 = prof_event(m);
+    if (!store)
+      launch_tet_sigma(m, list, count, s);
+    else if (mixed)
+      launch_tet_grad_mixed(m, list, count, elastic_weight(m), s);
+    else
+      launch_tet_grad_f64(m, x, list, count, elastic_weight(m), s);
+    prof_close(m, P_TET, e0, count > 0 ? 1 : 0);
+  }
   e0 = prof_event(m);
-  if (p == CC_PREC_FP64)
-    launch_rows_f64(m, x, xt, elastic_weight(m), s);
-  else
+  if (!store)
+    launch_rows_from_positions(m, mixed, x, xt, s);
+  else if (mixed)
     launch_rows_mixed(m, elastic_weight(m), s);
+  else
+    launch_rows_f64(m, x, xt, elastic_weight(m), s);
   prof_close(m, P_GATHER, e0, 1);
 }
 
@@ -403,13 +420,13 @@ void cc_destroy_mesh(cc_mesh* m) {
   drop_graph(*m);
   for (cudaEvent_t e : m->prof.pool) cudaEventDestroy(e);
   auto rel = [](auto& b) { b.release(); };
-  rel(m->d_tets); rel(m->d_tslot); rel(m->d_Bm); rel(m->d_Bm_df); rel(m->d_Bm32); rel(m->d_vol); rel(m->d_mat64); rel(m->d_matdf); rel(m->d_vert_mesh);
+  rel(m->d_tets); rel(m->d_tslot); rel(m->d_Bm); rel(m->d_Bm_df); rel(m->d_vol); rel(m->d_mat64); rel(m->d_matdf); rel(m->d_vert_mesh);
   rel(m->d_mesh_fptr); rel(m->d_mesh_active); rel(m->d_mesh_ones); rel(m->d_mesh_gsq); rel(m->d_volw); rel(m->d_volw32); rel(m->d_volw_df); rel(m->d_mass);
   rel(m->d_mass32); rel(m->d_mass_df);
   rel(m->d_pinned); rel(m->d_vt_ptr); rel(m->d_nbr_ptr); rel(m->d_nbr_idx); rel(m->d_vt_tet); rel(m->d_vt_corner);
   rel(m->d_up_ptr); rel(m->d_up_col); rel(m->d_rs_ptr); rel(m->d_rs_src); rel(m->d_free_rows); rel(m->d_row_hdr);
   rel(m->d_color); rel(m->d_cv_idx); rel(m->d_tl); rel(m->d_all_tets); rel(m->d_sup_ptr); rel(m->d_sup_idx); rel(m->d_smap_ptr);
-  rel(m->d_smap8); rel(m->d_smap16); rel(m->d_vt_ids);
+  rel(m->d_smap8); rel(m->d_smap16);
   rel(m->f64.gcon); rel(m->f64.hten); rel(m->f64.g); rel(m->f64.cpl); rel(m->f64.bsr); rel(m->f64.U);
   rel(m->mx.gcon); rel(m->mx.hten); rel(m->mx.cpl); rel(m->mx.g_hi); rel(m->mx.g_lo); rel(m->mx.bsr); rel(m->mx.U);
   rel(m->mx.x_hi); rel(m->mx.x_lo); rel(m->mx.xt_hi); rel(m->mx.xt_lo);
@@ -1120,7 +1137,7 @@ cc_status cc_autotune(cc_mesh* m, const double* x, const double* xt, cc_precisio
           out->variant_ms[v] = 0.0;
           m->rows_build = (v >> 1) != 0;
           m->fused_condense = (v & 1) != 0;
-          if (m->rows_build && !(p == CC_PREC_MIXED && rows_from_positions(*m))) continue;  // not applicable
+          if (m->rows_build && !rows_from_positions(*m)) continue;  // not applicable
           ensure_state(*m, p);
           drop_graph(*m);
           out->variant_ms[v] = time_sweeps();
@@ -1214,7 +1231,9 @@ cc_status cc_set_sweep_variant(cc_mesh* m, int32_t rows_from_positions, int32_t 
     if (rows_from_positions >= 0) m->rows_build = rows_from_positions != 0;
     if (fused_condense >= 0) m->fused_condense = fused_condense != 0;
     drop_graph(*m);
-    if (m->mx.gcon.p) ensure_state(*m, CC_PREC_MIXED);  // allocates the per-tet store if the gather path is back
+    // what the chosen row build needs (the per-tet store or the per-tet sigma)
+    if (m->mx.g_hi.p) ensure_state(*m, CC_PREC_MIXED);
+    if (m->f64.g.p) ensure_state(*m, CC_PREC_FP64);
   })
 }
 

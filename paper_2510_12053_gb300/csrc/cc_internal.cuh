@@ -120,6 +120,7 @@ struct StateF64 {
 struct StateMixed {
   DBuf<float2> gcon;  // [4T][3]   float-float (hi, lo)
   DBuf<float> hten;   // [T][kTetStore]
+  DBuf<float4> rec;   // [T] (sigma hi, sigma lo, c1, 0) of every tet (rows formed from the positions)
   DBuf<float> g_hi;   // [n][3]
   DBuf<float> g_lo;   // [n][3]
   DBuf<float> bsr;    // [nnz_up][12]
@@ -160,7 +161,7 @@ struct Mesh {
   int tune_couple_row_lanes = 4;  // threads per block row in the coupling kernel (1, 2, 4, 8)
   int tune_gather_wpb = 4;        // warps (rows) per block in the row gather
   bool fused_condense = false;    // the coupling kernel's last CTA of every 32 vertices condenses them
-  bool rows_build = false;        // mixed stable Neo-Hookean rows formed from the positions (k_row_build)
+  bool rows_build = true;         // stable Neo-Hookean rows formed from the positions (kernels_rows.cu)
   int64_t n = 0, T = 0, n_free = 0, nnzb = 0;
   int32_t max_valence = 0;
   double E = 0, nu = 0, rho = 0, mu = 0, lam_hat = 0, h = 0;
@@ -214,8 +215,6 @@ struct Mesh {
   DBuf<int4> d_tslot;        // [T] global (vertex, slot) entry of each corner
   DBuf<double> d_Bm;         // [T][9] D_m^{-1}, row-major (row c = shape vector of corner c+1)
   DBuf<float2> d_Bm_df;      // [T][9] float-float copy
-  DBuf<float> d_Bm32;        // [T][9]
-  DBuf<float> d_Bm32p;       // [T][3][4] rows padded to four (row build)
   DBuf<double> d_vol;        // [T]
   DBuf<double2> d_mat64;     // [T] (mu, lam_hat) of the tet's material
   DBuf<float4> d_matdf;      // [T] (mu hi, mu lo, lam_hat hi, lam_hat lo)
@@ -235,7 +234,6 @@ struct Mesh {
   DBuf<int32_t> d_up_col;    // [nnz_up]
   DBuf<int32_t> d_rs_ptr;    // [nnz_up+1] sources of each upper block (free rows)
   DBuf<int32_t> d_rs_src;    // per-tet store offset of each source, bit 31 = transpose
-  DBuf<uint16_t> d_rs_loc;   // the same sources as row-local codes k * 4 + w (row build)
   DBuf<int32_t> d_free_rows; // free vertices, ascending
   DBuf<int4> d_row_hdr;      // [2 n_free] row gather records: (j, p0, nup, rb), (rcount, e0, val, 0)
   DBuf<int32_t> d_color;     // [n]
@@ -254,7 +252,21 @@ struct Mesh {
   DBuf<int64_t> d_smap_ptr;  // [n+1]
   DBuf<uint8_t> d_smap8;
   DBuf<uint16_t> d_smap16;
-  DBuf<int4> d_vt_ids;       // [4T] vertex ids of the tet at each (vertex, slot) entry
+  // rows formed from the positions (kernels_rows.cu; stable Neo-Hookean)
+  bool rows_ok = false;      // the mesh fits that kernel (build_row_data)
+  int32_t max_ring = 0;      // most 1-ring neighbours of a vertex
+  float len_scale = 1.0f;    // power of two that brings the mean edge near 1 (mixed path)
+  DBuf<int4> d_row_hdr2;     // [2 n_free] (j, first upper block, upper blocks, first ring entry),
+                             //            (ring entries, first vertex-tet entry, entries, first block row)
+  DBuf<uint32_t> d_loc;      // [4T] ring slots of an entry's three other corners, a byte each
+  DBuf<double2> d_tc64;      // [T] (c1, c0): sigma = c1 det + c0
+  DBuf<float4> d_tcdf;       // [T] the same in scaled lengths, float-float
+  DBuf<double> d_ring_m64;   // [ring entries] m_jl
+  DBuf<float2> d_ring_mdf;   // [ring entries] float-float copy
+  DBuf<double> d_row_diag64; // [n_free] -sum_l m_jl (+ mass)
+  DBuf<float> d_row_diag32;
+  DBuf<uint4> d_codes8;      // [nnz_up] first eight source codes of every off-diagonal upper block
+  DBuf<uint16_t> d_rs_code;  // all source codes, in the order of d_rs_src
   DBuf<double> d_Xrest;      // [3][n] rest positions (uploaded on first use)
   bool rot_active = false;   // the current sweep uses corotated bases
 
@@ -295,10 +307,13 @@ __device__ __forceinline__ void pdl_entry() {
 
 bool pdl_enabled();  // true when CC_GB300_PDL is set in the environment (default: ordinary launches)
 
-// The mixed path of the stable Neo-Hookean material forms its float32 block
-// rows from the positions (k_row_build) instead of a per-tet Hessian store;
-// the float64 path and Fixed Corotational keep the store (FCR's blocks need
-// the polar rotation, too costly to form four times per tet).
+// Shared memory one CTA of the row kernel may take.
+constexpr size_t kRowsSmemMax = 200 * 1024;
+
+// Stable Neo-Hookean block rows are formed from the positions instead of a
+// per-tet Hessian store (kernels_rows.cu); Fixed Corotational keeps the store
+// (its blocks need the polar rotation, too costly to form four times per tet),
+// and so do meshes whose rows do not fit that kernel.
 // The coupling kernel condenses its vertices itself (one launch per colour
 // for the local solves) unless switched off or with the one-warp coupling kernel.
 inline bool fused_local_solve(const Mesh& m, cc_update upd) {
@@ -306,7 +321,7 @@ inline bool fused_local_solve(const Mesh& m, cc_update upd) {
 }
 
 inline bool rows_from_positions(const Mesh& m) {
-  return m.rows_build && m.model == CC_MODEL_SNH && m.max_valence <= 64;
+  return m.rows_build && m.rows_ok;
 }
 
 template <typename... KArgs, typename... Args>
@@ -347,6 +362,11 @@ struct SweepCounters {
 void launch_tet_grad_f64(Mesh& m, const double* x, const int32_t* list, int64_t count, double weight,
                          cudaStream_t s);
 void launch_tet_grad_mixed(Mesh& m, const int32_t* list, int64_t count, double weight, cudaStream_t s);
+// the same without the store: per-tet sigma (mixed), then rows from the positions
+void launch_tet_sigma(Mesh& m, const int32_t* list, int64_t count, cudaStream_t s);
+void launch_rows_from_positions(Mesh& m, bool mixed, const double* x, const double* xt, cudaStream_t s);
+// rest data of those rows (volw: per-tet volume times the elastic weight)
+void build_row_data(Mesh& m, const std::vector<double>& volw);
 // phase B: gradient and upper Hessian block rows of every free vertex
 void launch_rows_f64(Mesh& m, const double* x, const double* xt, double weight, cudaStream_t s);
 void launch_rows_mixed(Mesh& m, double weight, cudaStream_t s);

@@ -417,8 +417,12 @@ void build_supports(Mesh& m, int32_t k) {
 void hessian_f64_at(Mesh& m, const double* x) {
   cudaStream_t s = m.stream;
   const double w = m.h > 0.0 ? m.h * m.h : 1.0;
-  launch_tet_grad_f64(m, x, m.d_all_tets.p, m.n_active_tets, w, s);
-  launch_rows_f64(m, x, x, w, s);
+  if (rows_from_positions(m)) {
+    launch_rows_from_positions(m, false, x, x, s);
+  } else {
+    launch_tet_grad_f64(m, x, m.d_all_tets.p, m.n_active_tets, w, s);
+    launch_rows_f64(m, x, x, w, s);
+  }
   CCG_CUDA(cudaStreamSynchronize(s));
 }
 

@@ -151,13 +151,9 @@ void build_topology(Mesh& m) {
   //      per-tet Hessian store (kTetStore values per tet; a diagonal pair,
   //      cj == w, is stored as its upper triangle), bit 31 set when the
   //      stored block must be transposed (cj > w).  Ascending slot order.
-  //      The same sources also get a row-local code k * 4 + w (k = the
-  //      tet's position in the row's vertex-tet list, w = the corner of l in
-  //      it) for the row build, which forms K_{cj,w} itself.
   static const int kPair[4][4] = {{0, 1, 2, 3}, {1, 4, 5, 6}, {2, 5, 7, 8}, {3, 6, 8, 9}};
   std::vector<int32_t> rs_ptr(m.nnz_up + 1, 0);
   std::vector<int32_t> rs_src;
-  std::vector<uint16_t> rs_loc;
   for (int64_t v = 0; v < n; ++v) {
     const int64_t p0 = m.up_ptr[v], p1 = m.up_ptr[v + 1];
     if (m.pinned[v]) {
@@ -174,7 +170,6 @@ void build_topology(Mesh& m) {
           if (tv[w] == col) {
             const uint32_t off = (uint32_t)(t * kTetStore + tet_pair_offset(kPair[cj][w]));
             rs_src.push_back((int32_t)(off | (cj > w ? 0x80000000u : 0u)));
-            rs_loc.push_back((uint16_t)(((e - m.vt_ptr[v]) << 2) | w));
           }
       }
       rs_ptr[p + 1] = (int32_t)rs_src.size();
@@ -204,12 +199,9 @@ void build_topology(Mesh& m) {
 
   // ---- upload
   std::vector<float2> Bm_df(9 * T);
-  std::vector<float> Bm32(9 * T), Bm32p(12 * T, 0.0f);
   for (int64_t k = 0; k < 9 * T; ++k) {
     float hi = (float)Bm[k];
     Bm_df[k] = make_float2(hi, (float)(Bm[k] - (double)hi));
-    Bm32[k] = hi;
-    Bm32p[12 * (k / 9) + 4 * ((k % 9) / 3) + k % 3] = hi;  // rows padded to four for 16-byte loads
   }
   auto to32 = [&](const std::vector<int64_t>& a) {
     std::vector<int32_t> r(a.size());
@@ -220,8 +212,6 @@ void build_topology(Mesh& m) {
   m.d_tslot.upload(reinterpret_cast<const int4*>(tslot.data()), T, s);
   m.d_Bm.upload(Bm, s);
   m.d_Bm_df.upload(Bm_df, s);
-  m.d_Bm32.upload(Bm32, s);
-  m.d_Bm32p.upload(Bm32p, s);
   m.d_vol.upload(vol, s);
   {
     std::vector<double2> m64(T);
@@ -236,9 +226,9 @@ void build_topology(Mesh& m) {
     m.d_matdf.upload(mdf, s);
     CCG_CUDA(cudaStreamSynchronize(s));
   }
+  std::vector<double> vw(T);
   {
     const double w = m.h > 0.0 ? m.h * m.h : 1.0;
-    std::vector<double> vw(T);
     std::vector<float> vw32(T);
     std::vector<float2> vwdf(T);
     for (int64_t t = 0; t < T; ++t) {
@@ -272,7 +262,6 @@ void build_topology(Mesh& m) {
   m.d_up_col.upload(m.up_col, s);
   m.d_rs_ptr.upload(rs_ptr, s);
   m.d_rs_src.upload(rs_src, s);
-  m.d_rs_loc.upload(rs_loc, s);
   m.d_free_rows.upload(free_rows, s);
   {
     // per free row, what the row gather needs first, in one 32-byte record:
@@ -323,13 +312,7 @@ void build_topology(Mesh& m) {
     m.d_mesh_alpha.alloc(B);
     CCG_CUDA(cudaStreamSynchronize(s));
   }
-  {
-    std::vector<int32_t> ids(16 * T);
-    for (int64_t e = 0; e < 4 * T; ++e)
-      for (int c = 0; c < 4; ++c) ids[4 * e + c] = m.tets[4 * (int64_t)m.vt_tet[e] + c];
-    m.d_vt_ids.upload(reinterpret_cast<const int4*>(ids.data()), 4 * T, s);
-    CCG_CUDA(cudaStreamSynchronize(s));
-  }
+  build_row_data(m, vw);
   CCG_CUDA(cudaStreamSynchronize(s));  // host vectors above go out of scope
 }
 
