@@ -64,7 +64,7 @@ void ensure_state(Mesh& m, cc_precision p) {
   }
   if (p == CC_PREC_FP64) {
     // the per-tet store exists only where the rows are gathered from it
-    if (!rows_from_positions(m) && !m.f64.hten.p) {
+    if (!(rows_from_positions(m, false) && bases_from_positions(m)) && !m.f64.hten.p) {
       m.f64.gcon.alloc(3 * ne);
       m.f64.hten.alloc(kTetStore * (size_t)m.T);
     }
@@ -89,7 +89,7 @@ void ensure_state(Mesh& m, cc_precision p) {
       CCG_CUDA(cudaMemsetAsync(m.mx.xt_hi.p, 0, m.n * sizeof(float4), s));
       CCG_CUDA(cudaMemsetAsync(m.mx.xt_lo.p, 0, m.n * sizeof(float4), s));
     }
-    if (rows_from_positions(m)) {
+    if (rows_from_positions(m, true)) {
       if (!m.mx.rec.p) {
         m.mx.rec.alloc(m.T);
         CCG_CUDA(cudaMemsetAsync(m.mx.rec.p, 0, m.T * sizeof(float4), s));
@@ -165,7 +165,7 @@ double elastic_weight(const Mesh& m) { return m.h > 0.0 ? m.h * m.h : 1.0; }
 // Re-evaluates the per-tet derivatives for a tet list and re-gathers g, H.
 void refresh(Mesh& m, cc_precision p, const double* x, const double* xt, const int32_t* list, int64_t count) {
   cudaStream_t s = m.stream;
-  const bool store = !rows_from_positions(m), mixed = p == CC_PREC_MIXED;
+  const bool mixed = p == CC_PREC_MIXED, store = !rows_from_positions(m, mixed);
   int e0;
   if (store || mixed) {  // float64 rows from the positions need no per-tet pass
     e0 = prof_event(m);
@@ -1131,19 +1131,20 @@ cc_status cc_autotune(cc_mesh* m, const double* x, const double* xt, cc_precisio
     try {
       // sweep variant first, at the current launch shapes
       {
-        const bool rb0 = m->rows_build, fc0 = m->fused_condense;
+        const int rb0 = m->rows_build;
+        const bool fc0 = m->fused_condense;
         int best_v = -1;
         for (int v = 0; v < 4; ++v) {
           out->variant_ms[v] = 0.0;
-          m->rows_build = (v >> 1) != 0;
+          m->rows_build = v >> 1;
           m->fused_condense = (v & 1) != 0;
-          if (m->rows_build && !rows_from_positions(*m)) continue;  // not applicable
+          if (m->rows_build && !rows_from_positions(*m, p == CC_PREC_MIXED)) continue;  // not applicable
           ensure_state(*m, p);
           drop_graph(*m);
           out->variant_ms[v] = time_sweeps();
           if (best_v < 0 || out->variant_ms[v] < out->variant_ms[best_v]) best_v = v;
         }
-        m->rows_build = best_v >= 0 ? (best_v >> 1) != 0 : rb0;
+        m->rows_build = best_v >= 0 ? best_v >> 1 : rb0;
         m->fused_condense = best_v >= 0 ? (best_v & 1) != 0 : fc0;
         ensure_state(*m, p);
       }
@@ -1200,7 +1201,7 @@ cc_status cc_autotune(cc_mesh* m, const double* x, const double* xt, cc_precisio
     out->couple_threads = m->tune_couple_threads;
     out->couple_row_lanes = m->tune_couple_row_lanes;
     out->gather_warps = m->tune_gather_wpb;
-    out->rows_from_positions = m->rows_build ? 1 : 0;
+    out->rows_from_positions = rows_from_positions(*m, p == CC_PREC_MIXED) ? 1 : 0;
     out->fused_condense = m->fused_condense ? 1 : 0;
   })
 }
@@ -1228,7 +1229,7 @@ cc_status cc_set_sweep_variant(cc_mesh* m, int32_t rows_from_positions, int32_t 
     CCG_CHECK(m, CC_ERR_INVALID_ARG, "mesh is NULL");
     CCG_CHECK(rows_from_positions >= -1 && rows_from_positions <= 1 && fused_condense >= -1 && fused_condense <= 1,
               CC_ERR_INVALID_ARG, "variant switches are 1 (on), 0 (off) or -1 (keep)");
-    if (rows_from_positions >= 0) m->rows_build = rows_from_positions != 0;
+    if (rows_from_positions >= 0) m->rows_build = rows_from_positions;
     if (fused_condense >= 0) m->fused_condense = fused_condense != 0;
     drop_graph(*m);
     // what the chosen row build needs (the per-tet store or the per-tet sigma)

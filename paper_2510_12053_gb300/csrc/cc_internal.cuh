@@ -161,7 +161,7 @@ struct Mesh {
   int tune_couple_row_lanes = 4;  // threads per block row in the coupling kernel (1, 2, 4, 8)
   int tune_gather_wpb = 4;        // warps (rows) per block in the row gather
   bool fused_condense = false;    // the coupling kernel's last CTA of every 32 vertices condenses them
-  bool rows_build = true;         // stable Neo-Hookean rows formed from the positions (kernels_rows.cu)
+  int rows_build = -1;            // rows formed from the positions (kernels_rows.cu): 1, 0, -1 by rows_from_positions
   int64_t n = 0, T = 0, n_free = 0, nnzb = 0;
   int32_t max_valence = 0;
   double E = 0, nu = 0, rho = 0, mu = 0, lam_hat = 0, h = 0;
@@ -320,9 +320,20 @@ inline bool fused_local_solve(const Mesh& m, cc_update upd) {
   return upd != CC_UPDATE_CD && m.fused_condense && m.tune_couple_threads != 32;
 }
 
-inline bool rows_from_positions(const Mesh& m) {
-  return m.rows_build && m.rows_ok;
+// A dynamic mesh's float32 path keeps the store, and the slot-map coupling
+// kernel, unless switched on: a step returns v = (x_new - x_old) / h, which
+// shows the float32 rounding of the updates at full relative size (1e-7),
+// where positions show it four to five digits lower; so its sums keep the order
+// they have always had, and a step its bits.
+inline bool mixed_dynamic(const Mesh& m, bool mixed) { return mixed && m.h > 0.0; }
+
+inline bool rows_from_positions(const Mesh& m, bool mixed) {
+  return m.rows_ok && (m.rows_build < 0 ? !mixed_dynamic(m, mixed) : m.rows_build != 0);
 }
+
+// The float64 Hessian that bases are built from: a dynamic mesh's keeps the
+// store with its float32 path (whose float32 copies of the bases it rounds).
+inline bool bases_from_positions(const Mesh& m) { return rows_from_positions(m, m.h > 0.0); }
 
 template <typename... KArgs, typename... Args>
 void pdl_launch(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args&&... args) {

@@ -417,7 +417,7 @@ void build_supports(Mesh& m, int32_t k) {
 void hessian_f64_at(Mesh& m, const double* x) {
   cudaStream_t s = m.stream;
   const double w = m.h > 0.0 ? m.h * m.h : 1.0;
-  if (rows_from_positions(m)) {
+  if (bases_from_positions(m)) {
     launch_rows_from_positions(m, false, x, x, s);
   } else {
     launch_tet_grad_f64(m, x, m.d_all_tets.p, m.n_active_tets, w, s);
