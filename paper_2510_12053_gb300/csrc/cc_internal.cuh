@@ -420,6 +420,9 @@ void hessian_f64_at(Mesh& m, const double* x);
 // float32 factor + float64 refinement where the patch fits (<= 192 unknowns),
 // float64 Cholesky otherwise; returns the patches that were not positive
 // definite (their bases untouched), or throws when throw_on_fail.
+constexpr int kPmMaxN = 192;  // unknowns of the largest such patch (kernels_patch.cu)
+void launch_patch_basis_mixed(Mesh& m, const int32_t* d_verts, int64_t count, int32_t* redo, int32_t* n_redo,
+                              cudaStream_t s);
 int64_t patch_solves(Mesh& m, const int32_t* d_verts, int64_t count, bool throw_on_fail);
 int64_t rebuild_bases_at(Mesh& m, const double* x);
 // Eq. 5 residuals of the float64 bases of a device vertex list (mlp.cu)
