@@ -96,6 +96,9 @@ constexpr int kTetStore = 80;
 // copies a vertex's map in 4-byte words from the word holding its first code,
 // which reads up to 3 codes past the map's end.
 constexpr int kSlotMapSlack = 8;
+// Fields of a pair-list entry (Mesh::d_pairs).
+constexpr int kPairMaxSup = 1020, kPairMaxRow = 4095;
+constexpr uint32_t kPairSelf = 1023;
 constexpr bool tet_pair_is_diag(int pair) { return pair == 0 || pair == 4 || pair == 7 || pair == 9; }
 // first value of a pair's block in the tet's record
 constexpr int tet_pair_offset(int pair) {
@@ -252,6 +255,16 @@ struct Mesh {
   DBuf<int64_t> d_smap_ptr;  // [n+1]
   DBuf<uint8_t> d_smap8;
   DBuf<uint16_t> d_smap16;
+  // Pair lists of the float32 coupling kernel (k_couple_pairs): for free vertex
+  // i, the blocks (j, l), j < l, of the support's upper rows, then the ns
+  // blocks that couple a support row with i.  An entry is
+  // row slot | column slot << 10 | place in the row << 20; the slot of i is
+  // |S_i|, and kPairSelf as column slot marks a block (j, i) of a support row.
+  // Empty when a support or a row does not fit the fields.
+  bool pairs_ok = false;
+  DBuf<int4> d_pair_hdr;       // [2n] (first support entry, |S_i|, pairs, ns), (list start lo, hi, first block of row i, 0)
+  DBuf<int32_t> d_sup_row;     // [support_total] first upper block of every support vertex's row
+  DBuf<uint32_t> d_pairs;
   // rows formed from the positions (kernels_rows.cu; stable Neo-Hookean)
   bool rows_ok = false;      // the mesh fits that kernel (build_row_data)
   int32_t max_ring = 0;      // most 1-ring neighbours of a vertex

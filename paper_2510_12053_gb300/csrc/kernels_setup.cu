@@ -304,7 +304,115 @@ __global__ void k_slot_maps(const int32_t* __restrict__ rows, int64_t nrows, con
     base += __shfl_sync(0xffffffffu, incl, 31);
   }
 }
+
+// Pair lists (Mesh::d_pairs), one warp per free vertex v, in two passes:
+// kFill false counts the vertex's pairs and blocks with v itself (counts[w]),
+// true writes them in row order at the header's start, first the pairs.
+// Lane r takes row r of a 32-row chunk (rows 0..m-1 = S_v, row m = v).
+template <bool kFill>
+__global__ void k_pair_lists(const int32_t* __restrict__ rows, int64_t nrows, const int32_t* __restrict__ sup_ptr,
+                             const int32_t* __restrict__ sup_idx, const int32_t* __restrict__ up_ptr,
+                             const int32_t* __restrict__ up_col, int2* __restrict__ counts,
+                             const int4* __restrict__ hdr, int32_t* __restrict__ sup_row,
+                             uint32_t* __restrict__ list) {
+  const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (w >= nrows) return;  // whole warps leave together
+  const int v = rows[w];
+  const int s0 = sup_ptr[v], m = sup_ptr[v + 1] - s0;
+  const int32_t* S = sup_idx + s0;
+  uint32_t *pairs = nullptr, *self = nullptr;
+  if (kFill) {
+    const int4 a = hdr[2 * (int64_t)v], b = hdr[2 * (int64_t)v + 1];
+    pairs = list + ((int64_t)(uint32_t)b.x | ((int64_t)b.y << 32));
+    self = pairs + a.z;
+  }
+  int npair = 0, nself = 0;
+  for (int r0 = 0; r0 <= m; r0 += 32) {
+    const int r = r0 + lane;
+    int p0 = 0, len = 0;
+    if (r <= m) {
+      const int j = r < m ? S[r] : v;
+      p0 = up_ptr[j];
+      len = up_ptr[j + 1] - p0;
+      if (kFill && r < m) sup_row[s0 + r] = p0;
+    }
+    // what one block of the lane's row is: 1 a pair, 2 a block with v, 0 neither
+    auto kind = [&](int q, uint32_t* col) {
+      const int l = up_col[p0 + q];
+      if (l == v) {
+        *col = kPairSelf;
+        return 2;
+      }
+      const int t = find_in_sorted(S, m, l);
+      *col = (uint32_t)t;
+      return t < 0 ? 0 : r < m ? 1 : 2;
+    };
+    int cp = 0, cs = 0;
+    uint32_t col;
+    for (int q = 1; q < len; ++q) {
+      const int k = kind(q, &col);
+      cp += k == 1;
+      cs += k == 2;
+    }
+    int ip = cp, is = cs;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int tp = __shfl_up_sync(0xffffffffu, ip, o), ts = __shfl_up_sync(0xffffffffu, is, o);
+      if (lane >= o) {
+        ip += tp;
+        is += ts;
+      }
+    }
+    if (kFill) {
+      int wp = npair + ip - cp, ws = nself + is - cs;
+      for (int q = 1; q < len; ++q) {
+        const int k = kind(q, &col);
+        const uint32_t e = (uint32_t)r | (col << 10) | ((uint32_t)q << 20);
+        if (k == 1) pairs[wp++] = e;
+        if (k == 2) self[ws++] = e;
+      }
+    }
+    npair += __shfl_sync(0xffffffffu, ip, 31);
+    nself += __shfl_sync(0xffffffffu, is, 31);
+  }
+  if (!kFill && lane == 0) counts[w] = make_int2(npair, nself);
+}
 }  // namespace
+
+// Pair lists of the current supports; the host places the vertices' lists.
+static void build_pair_lists(Mesh& m) {
+  cudaStream_t s = m.stream;
+  m.pairs_ok = false;
+  m.d_pairs.release();
+  if (m.sup_max > kPairMaxSup || m.max_up > kPairMaxRow || m.n_free <= 0) return;
+  const int64_t nf = m.n_free, total = m.sup_ptr[m.n];
+  const unsigned grid = (unsigned)((nf * 32 + 255) / 256);
+  DBuf<int2> d_counts;
+  d_counts.alloc(nf);
+  k_pair_lists<false><<<grid, 256, 0, s>>>(m.d_free_rows.p, nf, m.d_sup_ptr.p, m.d_sup_idx.p, m.d_up_ptr.p,
+                                           m.d_up_col.p, d_counts.p, nullptr, nullptr, nullptr);
+  std::vector<int2> counts(nf);
+  CCG_CUDA(cudaMemcpyAsync(counts.data(), d_counts.p, nf * sizeof(int2), cudaMemcpyDeviceToHost, s));
+  CCG_CUDA(cudaStreamSynchronize(s));
+  std::vector<int4> hdr(2 * m.n, make_int4(0, 0, 0, 0));
+  int64_t at = 0, w = 0;
+  for (int64_t v = 0; v < m.n; ++v) {
+    if (m.pinned[v]) continue;
+    const int2 c = counts[w++];
+    hdr[2 * v] = make_int4((int)m.sup_ptr[v], (int)(m.sup_ptr[v + 1] - m.sup_ptr[v]), c.x, c.y);
+    hdr[2 * v + 1] = make_int4((int)(uint32_t)(at & 0xffffffff), (int)(at >> 32), (int)m.up_ptr[v], 0);
+    at += c.x + c.y;
+  }
+  m.d_pair_hdr.upload(hdr, s);
+  m.d_sup_row.alloc(total);
+  m.d_pairs.alloc(at);
+  k_pair_lists<true><<<grid, 256, 0, s>>>(m.d_free_rows.p, nf, m.d_sup_ptr.p, m.d_sup_idx.p, m.d_up_ptr.p,
+                                          m.d_up_col.p, nullptr, m.d_pair_hdr.p, m.d_sup_row.p, m.d_pairs.p);
+  CCG_CUDA(cudaGetLastError());
+  CCG_CUDA(cudaStreamSynchronize(s));  // the host vectors above go out of scope
+  m.pairs_ok = true;
+}
 
 // Slot maps of the current supports (cc_build_subspace / cc_set_subspace),
 // built on the device from the uploaded supports and upper block pattern.
@@ -312,6 +420,7 @@ __global__ void k_slot_maps(const int32_t* __restrict__ rows, int64_t nrows, con
 void build_slot_maps(Mesh& m) {
   const int64_t n = m.n;
   cudaStream_t s = m.stream;
+  build_pair_lists(m);
   m.smap_wide = m.sup_max >= 250;
   std::vector<int64_t> len(n, 0);
   const int nt = host_threads(n);

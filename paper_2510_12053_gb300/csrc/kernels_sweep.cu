@@ -696,6 +696,148 @@ void launch_couple_warp(Mesh& m, const int32_t* verts, int64_t count, const HT* 
   CCG_CUDA(cudaGetLastError());
 }
 
+// Float32 coupling products, one CTA per free vertex i of the list, from the
+// vertex's pair list (Mesh::d_pairs).  Three loops without divergence:
+//   support rows j      1/2 H_jj's share of Ht and U_j^T g_j, a row per thread;
+//   pairs (j, l), j < l of the support, a block per thread: M += U_j^T (H_jl U_l);
+//   blocks with i       A += H_ij U_j (stored as H_ji^T or H_ij), from thread
+//                       kThreads/2 on, where the last round of pairs is empty
+//                       more often;
+// and Ht = M + M^T.  Every entry says which block and which basis slots it
+// needs, so a thread's list entry, block row and basis rows are all known two
+// loads after the vertex number, and no thread walks blocks outside the support.
+template <int kThreads, int kUpd, bool kFuse>
+__global__ void __launch_bounds__(kThreads, 1024 / kThreads) k_couple_pairs(
+    const int32_t* __restrict__ verts, int64_t count, const int4* __restrict__ hdr,
+    const int32_t* __restrict__ sup_idx, const int32_t* __restrict__ sup_row, const float* __restrict__ U,
+    const uint32_t* __restrict__ list, const float* __restrict__ bsr, const float* __restrict__ g_hi, int sup_max,
+    const float* __restrict__ rot, float* __restrict__ cpl, CondenseArgs<float> ca) {
+  pdl_entry();
+  extern __shared__ __align__(16) unsigned char smem[];
+  float* Us = reinterpret_cast<float*>(smem);  // [m][3][4]
+  int* rstart = reinterpret_cast<int*>(smem + align16((size_t)sup_max * 12 * sizeof(float)));  // [m + 1]
+  constexpr int kWarps = kThreads / 32;
+  __shared__ float red[kWarps][18];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int i = verts[blockIdx.x];
+  const int4 ha = __ldg(hdr + 2 * (int64_t)i), hb = __ldg(hdr + 2 * (int64_t)i + 1);
+  const int s0 = ha.x, m = ha.y, np = ha.z, ns = ha.w;
+  const uint32_t* L = list + ((int64_t)(uint32_t)hb.x | ((int64_t)hb.y << 32));
+  uint32_t next = tid < np ? __ldg(L + tid) : 0u;
+  stage_basis<float, 12, 4>(Us, U, rot, sup_idx, s0, m, tid, kThreads);
+  for (int s = tid; s < m; s += kThreads) rstart[s] = __ldg(sup_row + s0 + s);
+  if (tid == 0) rstart[m] = hb.z;
+  float* out = cpl + (int64_t)blockIdx.x * 32;
+  if (tid < 9) out[18 + tid] = __ldg(bsr + (int64_t)hb.z * 12 + 4 * (tid / 3) + tid % 3);
+  __syncthreads();
+
+  float M[9], A[9], b[3] = {0, 0, 0};
+  mat3_zero(M);
+  mat3_zero(A);
+  for (int r = tid; r < m; r += kThreads) {
+    float H[9], Uj[9], T[9];
+    const int j = __ldg(sup_idx + s0 + r);
+    load_block(bsr, (int64_t)rstart[r], H);
+    load_slot(Us + 12 * r, Uj);
+    const float g0 = g_hi[3 * (int64_t)j], g1 = g_hi[3 * (int64_t)j + 1], g2 = g_hi[3 * (int64_t)j + 2];
+    mat3_zero(T);
+    mat3_mul_acc(H, Uj, T);
+#pragma unroll
+    for (int c = 0; c < 9; ++c) T[c] *= 0.5f;
+    mat3_tmul_acc(Uj, T, M);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) b[c] += Uj[c] * g0 + Uj[3 + c] * g1 + Uj[6 + c] * g2;
+  }
+  for (int e = tid; e < np; e += kThreads) {
+    const uint32_t w = next;
+    if (e + kThreads < np) next = __ldg(L + e + kThreads);
+    const int r = w & 1023, l = (w >> 10) & 1023;
+    float H[9], Ul[9], Uj[9], T[9];
+    load_block(bsr, (int64_t)(rstart[r] + (int)(w >> 20)), H);
+    load_slot(Us + 12 * l, Ul);
+    mat3_zero(T);
+    mat3_mul_acc(H, Ul, T);
+    load_slot(Us + 12 * r, Uj);
+    mat3_tmul_acc(Uj, T, M);
+  }
+  if (kUpd == CC_UPDATE_CC) {
+    for (int e = tid ^ (kThreads / 2); e < ns; e += kThreads) {
+      const uint32_t w = __ldg(L + np + e);
+      const int r = w & 1023, l = (w >> 10) & 1023;
+      const bool lower = l == (int)kPairSelf;  // stored as H_ji, j = row r of the support
+      float H[9], Uv[9];
+      load_block(bsr, (int64_t)(rstart[r] + (int)(w >> 20)), H);
+      load_slot(Us + 12 * (lower ? r : l), Uv);
+      if (lower) {
+        float t;
+        t = H[1]; H[1] = H[3]; H[3] = t;
+        t = H[2]; H[2] = H[6]; H[6] = t;
+        t = H[5]; H[5] = H[7]; H[7] = t;
+      }
+      mat3_mul_acc(H, Uv, A);
+    }
+  }
+
+  // the CTA's sums in a fixed order: sixteen values halved over the lanes
+  // (lane L ends with value (L >> 1) reversed in four bits), the last two by a
+  // butterfly each, then the warps' sums in order
+  float v[16] = {2.f * M[0], M[1] + M[3], M[2] + M[6], 2.f * M[4], M[5] + M[7], 2.f * M[8],
+                 A[0], A[1], A[2], A[3], A[4], A[5], A[6], A[7], A[8], b[0]};
+#pragma unroll
+  for (int o = 16, h = 8; h > 0; o >>= 1, h >>= 1) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int q = 0; q < h; ++q) {
+      const float keep = up ? v[q + h] : v[q], send = up ? v[q] : v[q + h];
+      v[q] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+  v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+  const float b1 = warp_sum(b[1]), b2 = warp_sum(b[2]);
+  const int mine = ((lane & 16) >> 1) | ((lane & 8) >> 1) | ((lane & 4) >> 1) | ((lane & 2) >> 1);
+  if constexpr (kWarps == 1) {
+    if ((lane & 1) == 0) out[mine] = v[0];
+    if (lane == 0) {
+      out[16] = b1;
+      out[17] = b2;
+    }
+  } else {
+    if ((lane & 1) == 0) red[warp][mine] = v[0];
+    if (lane == 0) {
+      red[warp][16] = b1;
+      red[warp][17] = b2;
+    }
+    __syncthreads();
+    if (tid < 18) {
+      float t = red[0][tid];
+#pragma unroll
+      for (int q = 1; q < kWarps; ++q) t += red[q][tid];
+      out[tid] = t;
+    }
+  }
+  if constexpr (kFuse) condense_group_tail<double, float, true, kUpd>(ca, 1e-12);
+}
+
+template <int kThreads, int kUpd>
+void launch_couple_pairs(Mesh& m, const int32_t* verts, int64_t count, const float* U, const float* bsr,
+                         const float* g_hi, float* cpl, const float* rot, const CondenseArgs<float>& ca, bool fuse,
+                         cudaStream_t s) {
+  const int supm = m.sup_max > 0 ? m.sup_max : 1;
+  const size_t smem = align16((size_t)supm * 12 * sizeof(float)) + align16((size_t)(supm + 1) * 4);
+  // the limit on supports is the one of the slot-map kernels, whichever kernel runs
+  CCG_CHECK(kThreads == 32 || cta_smem_bytes<float>(supm, m.smap_max, m.smap_wide ? 2 : 1, kThreads) <= 220 * 1024,
+            CC_ERR_INVALID_ARG, "support too large for the coupling kernel");
+  auto go = [&](auto kern) {
+    set_smem_limit(reinterpret_cast<const void*>(kern), smem);
+    pdl_launch(kern, (unsigned)count, kThreads, smem, s, verts, count, (const int4*)m.d_pair_hdr.p,
+               (const int32_t*)m.d_sup_idx.p, (const int32_t*)m.d_sup_row.p, U, (const uint32_t*)m.d_pairs.p, bsr,
+               g_hi, supm, rot, cpl, ca);
+  };
+  if (fuse) go(k_couple_pairs<kThreads, kUpd, true>);
+  else go(k_couple_pairs<kThreads, kUpd, false>);
+  CCG_CUDA(cudaGetLastError());
+}
+
 template <typename HT, bool kMixed, int kUpd>
 void launch_one(Mesh& m, const int32_t* verts, int64_t count, const HT* U, const HT* bsr, const double* g64,
                 const float* g_hi, const float* g_lo, HT* cpl, double* x, SweepCounters c, cudaStream_t s) {
@@ -714,7 +856,19 @@ void launch_one(Mesh& m, const int32_t* verts, int64_t count, const HT* U, const
       if constexpr (kMixed) rot = reinterpret_cast<const HT*>(m.mx.rot.p);
       else rot = reinterpret_cast<const HT*>(m.f64.rot.p);
     }
-    switch (m.tune_couple_threads) {
+    bool done = false;
+    if constexpr (kMixed) {
+      if (m.pairs_ok && !mixed_dynamic(m, kMixed)) {
+        done = true;
+        switch (m.tune_couple_threads) {
+          case 32: launch_couple_pairs<32, kUpd>(m, verts, count, U, bsr, g_hi, cpl, rot, cf, fuse, s); break;
+          case 64: launch_couple_pairs<64, kUpd>(m, verts, count, U, bsr, g_hi, cpl, rot, cf, fuse, s); break;
+          case 256: launch_couple_pairs<256, kUpd>(m, verts, count, U, bsr, g_hi, cpl, rot, cf, fuse, s); break;
+          default: launch_couple_pairs<128, kUpd>(m, verts, count, U, bsr, g_hi, cpl, rot, cf, fuse, s);
+        }
+      }
+    }
+    if (!done) switch (m.tune_couple_threads) {
       case 32: launch_couple_warp<HT, kMixed, kUpd>(m, verts, count, U, bsr, g64, g_hi, cpl, rot, s); break;
       case 64: launch_couple<HT, kMixed, kUpd, 64>(m, verts, count, U, bsr, g64, g_hi, cpl, rot, cf, fuse, s); break;
       case 256: launch_couple<HT, kMixed, kUpd, 256>(m, verts, count, U, bsr, g64, g_hi, cpl, rot, cf, fuse, s); break;
