@@ -168,10 +168,12 @@ struct Arith<double> {
   using V = double;
   static __device__ __forceinline__ V mk(double a) { return a; }
   static __device__ __forceinline__ V mkf(float a) { return (double)a; }
-  static __device__ __forceinline__ V add(V a, V b) { return a + b; }
-  static __device__ __forceinline__ V sub(V a, V b) { return a - b; }
-  static __device__ __forceinline__ V mul(V a, V b) { return a * b; }
-  static __device__ __forceinline__ V fma(V a, V b, V c) { return ::fma(a, b, c); }
+  // each rounds where it says (never contracted): kernels that split a vertex's
+  // algebra over lanes differently give the same bits
+  static __device__ __forceinline__ V add(V a, V b) { return __dadd_rn(a, b); }
+  static __device__ __forceinline__ V sub(V a, V b) { return __dsub_rn(a, b); }
+  static __device__ __forceinline__ V mul(V a, V b) { return __dmul_rn(a, b); }
+  static __device__ __forceinline__ V fma(V a, V b, V c) { return __fma_rn(a, b, c); }
   static __device__ __forceinline__ V div(V a, V b) { return a / b; }
   static __device__ __forceinline__ V neg(V a) { return -a; }
   static __device__ __forceinline__ bool gt(V a, V b) { return a > b; }
@@ -210,12 +212,12 @@ __device__ __forceinline__ bool sym3_adj(const typename Arith<T>::V* M, typename
   if (A::gt(m22, dmax)) dmax = m22;
   if (!A::gt(dmax, A::mkf(0.0f))) return false;
   const V thr = A::mul(rel, dmax);
-  const V c00 = A::sub(A::mul(m11, m22), A::mul(m21, m21));
-  const V c01 = A::sub(A::mul(m21, m20), A::mul(m10, m22));
-  const V c02 = A::sub(A::mul(m10, m21), A::mul(m11, m20));
-  const V c11 = A::sub(A::mul(m00, m22), A::mul(m20, m20));
-  const V c12 = A::sub(A::mul(m10, m20), A::mul(m00, m21));
-  const V c22 = A::sub(A::mul(m00, m11), A::mul(m10, m10));
+  const V c00 = A::fma(m11, m22, A::neg(A::mul(m21, m21)));
+  const V c01 = A::fma(m21, m20, A::neg(A::mul(m10, m22)));
+  const V c02 = A::fma(m10, m21, A::neg(A::mul(m11, m20)));
+  const V c11 = A::fma(m00, m22, A::neg(A::mul(m20, m20)));
+  const V c12 = A::fma(m10, m20, A::neg(A::mul(m00, m21)));
+  const V c22 = A::fma(m00, m11, A::neg(A::mul(m10, m10)));
   const V d3 = A::fma(m00, c00, A::fma(m10, c01, A::mul(m20, c02)));
   // pivots: p0 = m00, p1 = c22 / m00, p2 = d3 / c22
   if (!A::gt(m00, thr)) return false;

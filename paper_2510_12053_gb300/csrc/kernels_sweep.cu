@@ -295,7 +295,7 @@ __device__ __forceinline__ void condense_vertex(const CondenseArgs<HT>& c, int64
   double xn[3];
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    xn[a] = c.x[a * c.n + i] + d[a];
+    xn[a] = __dadd_rn(c.x[a * c.n + i], d[a]);
     c.x[a * c.n + i] = xn[a];
   }
   if (kMixed) {
@@ -303,6 +303,155 @@ __device__ __forceinline__ void condense_vertex(const CondenseArgs<HT>& c, int64
     c.x_hi[i] = make_float4(a0.hi, a1.hi, a2.hi, 0.f);
     c.x_lo[i] = make_float4(a0.lo, a1.lo, a2.lo, 0.f);
   }
+}
+
+// The condensation of condense_vertex with four lanes per vertex, lane r < 3
+// taking row r (lane 3 repeats row 2); the same roundings in the same order, so
+// the same bits.  The symmetric 3x3 inverses give each lane two cofactors and
+// one pivot test.  Lanes of a dead entry repeat the last one and write nothing.
+struct QuadSym3 {
+  double adj[6], det;  // cofactors (00 01 02 11 12 22)
+  bool ok;             // the pivot test
+};
+
+__device__ __forceinline__ QuadSym3 quad_sym3(const double* m /*00 10 11 20 21 22*/, double rel, int r, int base) {
+  using A = Arith<double>;
+  auto get = [&](double v, int src) { return __shfl_sync(0xffffffffu, v, base + src); };
+  const double m00 = m[0], m10 = m[1], m11 = m[2], m20 = m[3], m21 = m[4], m22 = m[5];
+  double dmax = m00;
+  if (A::gt(m11, dmax)) dmax = m11;
+  if (A::gt(m22, dmax)) dmax = m22;
+  const double thr = A::mul(rel, dmax);
+  // lane 0: c00, c01; lane 1: c02, c11; lane 2: c12, c22
+  const double u = A::fma(r == 0 ? m11 : m10, r == 0 ? m22 : r == 1 ? m21 : m20,
+                          A::neg(A::mul(r == 0 ? m21 : r == 1 ? m11 : m00, r == 1 ? m20 : m21)));
+  const double v = A::fma(r == 0 ? m21 : m00, r == 0 ? m20 : r == 1 ? m22 : m11,
+                          A::neg(A::mul(r == 1 ? m20 : m10, r == 0 ? m22 : r == 1 ? m20 : m10)));
+  QuadSym3 s;
+  s.adj[0] = get(u, 0); s.adj[1] = get(v, 0); s.adj[2] = get(u, 1);
+  s.adj[3] = get(v, 1); s.adj[4] = get(u, 2); s.adj[5] = get(v, 2);
+  s.det = A::fma(m00, s.adj[0], A::fma(m10, s.adj[1], A::mul(m20, s.adj[2])));
+  const bool pass = A::gt(r == 0 ? m00 : r == 1 ? s.adj[5] : s.det, r == 0 ? thr : A::mul(thr, r == 1 ? m00 : s.adj[5]));
+  const unsigned votes = __ballot_sync(0xffffffffu, pass) >> base;
+  s.ok = A::gt(dmax, 0.0) && (votes & 7u) == 7u;
+  return s;
+}
+
+template <typename HT, bool kMixed, int kUpd>
+__device__ __forceinline__ void condense_quad(const CondenseArgs<HT>& c, int64_t k, double rel) {
+  using Ar = Arith<double>;
+  const int lane = threadIdx.x & 31, base = lane & 28, r = min(lane & 3, 2);
+  auto get = [&](double v, int src) { return __shfl_sync(0xffffffffu, v, base + src); };
+  bool live = k < c.count;
+  if (!live) k = c.count - 1;
+  const int i = c.verts[k];
+  live = live && c.active[c.vert_mesh[i]] != 0;  // this mesh of the batch may have stopped
+  const HT* cp = c.cpl + k * 32;
+  double H[3], g;
+  {
+    const HT* h = kUpd == CC_UPDATE_CD ? c.bsr + (int64_t)c.up_ptr[i] * 12 + 4 * r : cp + 18 + 3 * r;
+#pragma unroll
+    for (int q = 0; q < 3; ++q) H[q] = (double)h[q];
+  }
+  if constexpr (!kMixed) g = c.g64[3 * (int64_t)i + r];
+  else g = Ar::add((double)c.g_hi[3 * (int64_t)i + r], (double)c.g_lo[3 * (int64_t)i + r]);
+  double dx = 0.0;
+  int fb = -1;
+  bool done = false;
+  if constexpr (kUpd != CC_UPDATE_CD) {
+    const bool empty = c.sup_ptr[i + 1] == c.sup_ptr[i];
+    const double tu = (double)cp[2 * r], tv = (double)cp[2 * r + 1];  // Ht (00 01 | 02 11 | 12 22)
+    const double b_r = (double)cp[15 + r];
+    const double t[6] = {get(tu, 0), get(tv, 0), get(tv, 1), get(tu, 1), get(tu, 2), get(tv, 2)};  // 00 10 11 20 21 22
+    double M[3], rhs;
+    bool reduced = true;
+    if constexpr (kUpd == CC_UPDATE_JGS2) {
+      M[0] = Ar::add(H[0], r == 0 ? t[0] : r == 1 ? t[1] : t[3]);
+      M[1] = Ar::add(H[1], r == 0 ? t[1] : r == 1 ? t[2] : t[4]);
+      M[2] = Ar::add(H[2], r == 0 ? t[3] : r == 1 ? t[4] : t[5]);
+      rhs = Ar::add(g, b_r);
+    } else {
+      const double b[3] = {get(b_r, 0), get(b_r, 1), get(b_r, 2)};
+      double A[3][3], Ao[3];
+#pragma unroll
+      for (int q = 0; q < 3; ++q) Ao[q] = (double)cp[6 + 3 * r + q];
+#pragma unroll
+      for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int q = 0; q < 3; ++q) A[a][q] = get(Ao[q], a);
+      const QuadSym3 s = quad_sym3(t, rel, r, base);
+      reduced = s.ok;
+      const double inv = Ar::div(1.0, s.det);
+      // each lane scales two of the six cofactors
+      const double su = Ar::mul(r == 0 ? s.adj[0] : r == 1 ? s.adj[2] : s.adj[4], inv);
+      const double sv = Ar::mul(r == 0 ? s.adj[1] : r == 1 ? s.adj[3] : s.adj[5], inv);
+      const double h00 = get(su, 0), h01 = get(sv, 0), h02 = get(su, 1), h11 = get(sv, 1), h12 = get(su, 2),
+                   h22 = get(sv, 2);
+      double W[3];
+      W[0] = Ar::fma(Ao[2], h02, Ar::fma(Ao[1], h01, Ar::mul(Ao[0], h00)));
+      W[1] = Ar::fma(Ao[2], h12, Ar::fma(Ao[1], h11, Ar::mul(Ao[0], h01)));
+      W[2] = Ar::fma(Ao[2], h22, Ar::fma(Ao[1], h12, Ar::mul(Ao[0], h02)));
+#pragma unroll
+      for (int q = 0; q < 3; ++q)
+        M[q] = Ar::sub(H[q], Ar::fma(W[2], A[q][2], Ar::fma(W[1], A[q][1], Ar::mul(W[0], A[q][0]))));
+      rhs = Ar::sub(g, Ar::fma(W[2], b[2], Ar::fma(W[1], b[1], Ar::mul(W[0], b[0]))));
+    }
+    const double m[6] = {get(M[0], 0), get(M[0], 1), get(M[1], 1), get(M[0], 2), get(M[1], 2), get(M[2], 2)};
+    const QuadSym3 s = quad_sym3(m, rel, r, base);
+    const double r0 = get(rhs, 0), r1 = get(rhs, 1), r2 = get(rhs, 2);
+    const double inv = Ar::neg(Ar::div(1.0, s.det));
+    dx = Ar::mul(inv, Ar::fma(r == 0 ? s.adj[0] : r == 1 ? s.adj[1] : s.adj[2], r0,
+                              Ar::fma(r == 0 ? s.adj[1] : r == 1 ? s.adj[3] : s.adj[4], r1,
+                                      Ar::mul(r == 0 ? s.adj[2] : r == 1 ? s.adj[4] : s.adj[5], r2))));
+    done = !empty && reduced && s.ok;
+    if (!done) fb = empty ? 0 : !reduced ? 1 : kUpd == CC_UPDATE_JGS2 ? 1 : 2;
+  }
+  bool bad = false;
+  if (__any_sync(0xffffffffu, live && !done)) {  // coordinate descent step: one Newton step on the vertex
+    const double m[6] = {get(H[0], 0), get(H[0], 1), get(H[1], 1), get(H[0], 2), get(H[1], 2), get(H[2], 2)};
+    const QuadSym3 s = quad_sym3(m, 0.0, r, base);
+    const double g0 = get(g, 0), g1 = get(g, 1), g2 = get(g, 2);
+    const double inv = Ar::neg(Ar::div(1.0, s.det));
+    const double cd = Ar::mul(inv, Ar::fma(r == 0 ? s.adj[0] : r == 1 ? s.adj[1] : s.adj[2], g0,
+                                           Ar::fma(r == 0 ? s.adj[1] : r == 1 ? s.adj[3] : s.adj[4], g1,
+                                                   Ar::mul(r == 0 ? s.adj[2] : r == 1 ? s.adj[4] : s.adj[5], g2))));
+    if (!done) {
+      dx = cd;
+      bad = !s.ok;
+    }
+  }
+  const unsigned finite = __ballot_sync(0xffffffffu, isfinite(dx)) >> base;
+  if (!live || (lane & 3) == 3) return;
+  if (bad || (finite & 7u) != 7u) {
+    if ((lane & 3) == 0) {
+      if (!bad && fb >= 0) atomicAdd(&c.fallback[fb], 1ull);
+      atomicOr(c.err, 1ull);
+    }
+    return;
+  }
+  if (fb >= 0 && (lane & 3) == 0) atomicAdd(&c.fallback[fb], 1ull);
+  const double xn = __dadd_rn(c.x[r * c.n + i], dx);
+  c.x[r * c.n + i] = xn;
+  if (kMixed) {
+    const df a = df_from_double(xn);
+    reinterpret_cast<float*>(c.x_hi + i)[r] = a.hi;
+    reinterpret_cast<float*>(c.x_lo + i)[r] = a.lo;
+  }
+}
+
+// Colours of at most this many vertices take four lanes a vertex.  The float64
+// pipe issues one warp instruction per sub-partition in about 61 cycles however
+// few lanes work, and a vertex alone in its lane takes about 250 of them: up to
+// 4 864 vertices (one four-lane warp for each of the 608 sub-partitions) the
+// shorter chain is what counts, beyond that the number of warps.  A mixed sweep
+// of the 8^3 cube (142 vertices a colour) 154 -> 140 us, three sweeps of a twisted
+// bar of 570 a colour 2.34 -> 2.21 ms; same bits.
+constexpr int64_t kCondenseQuadMax = 608 * 8;
+
+template <typename HT, bool kMixed, int kUpd>
+__global__ void __launch_bounds__(32) k_condense_quad(CondenseArgs<HT> c, double rel) {
+  pdl_entry();
+  condense_quad<HT, kMixed, kUpd>(c, (int64_t)blockIdx.x * 8 + (threadIdx.x >> 2), rel);
 }
 
 // Batched condensation, one list entry per thread: a warp condenses 32
@@ -880,6 +1029,11 @@ void launch_one(Mesh& m, const int32_t* verts, int64_t count, const HT* U, const
   // Eq. 11-12 stay in float64 in both precisions), one vertex per thread in
   // 32-thread blocks: a colour holds a few thousand vertices, so small blocks
   // spread the long per-vertex chains over every SM
+  if (count <= kCondenseQuadMax) {
+    pdl_launch(k_condense_quad<HT, kMixed, kUpd>, (unsigned)((count + 7) / 8), 32, 0, s, ca, 1e-12);
+    CCG_CUDA(cudaGetLastError());
+    return;
+  }
   constexpr int kCondenseThreads = 32;
   const unsigned grid = (unsigned)((count + kCondenseThreads - 1) / kCondenseThreads);
   pdl_launch(k_condense<double, HT, kMixed, kUpd>, grid, kCondenseThreads, 0, s, ca, 1e-12);
