@@ -310,40 +310,29 @@ __global__ void k_basis_residual(int nrows, const int32_t* __restrict__ rows, co
 // ---------------------------------------------------------------------------
 // Network kernels
 // ---------------------------------------------------------------------------
-// dst row b = src row idx[b] (BF16 rows of `cols` elements, 16-byte chunks).
-// Training minibatch rows: row b of step *step is idx[*step * B + b] (the
-// step counter lives on the device, so one captured step replays for all).
-__global__ void k_gather_rows_bf16(const bf16* __restrict__ src, int64_t lds, const int32_t* __restrict__ idx,
-                                   const int* __restrict__ step, int B, int chunks, bf16* __restrict__ dst,
-                                   int64_t ldd) {
-  const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (k >= (int64_t)B * chunks) return;
-  const int b = (int)(k / chunks), c = (int)(k % chunks);
-  const int32_t row = idx[(int64_t)*step * B + b];
-  reinterpret_cast<uint4*>(dst + (int64_t)b * ldd)[c] = reinterpret_cast<const uint4*>(src + (int64_t)row * lds)[c];
-}
-
-// vec = 4: cols, lds and ldd multiples of 4 and both bases 16-byte aligned
-// (float4 copies); else vec = 1.
-template <int vec>
-__global__ void k_gather_rows_f32(const float* __restrict__ src, int64_t lds, const int32_t* __restrict__ idx,
-                                  const int* __restrict__ step, int B, int cols, float* __restrict__ dst,
-                                  int64_t ldd) {
-  const int per = cols / vec;
-  const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (k >= (int64_t)B * per) return;
-  const int b = (int)(k / per), c = (int)(k % per) * vec;
-  const float* s = src + (int64_t)idx[(int64_t)*step * B + b] * lds + c;
-  float* d = dst + (int64_t)b * ldd + c;
-  if constexpr (vec == 4) *reinterpret_cast<float4*>(d) = *reinterpret_cast<const float4*>(s);
-  else *d = *s;
-}
-
-// end of a training step: the next step's number and beta^t
-__global__ void k_step_advance(int* __restrict__ step, double* __restrict__ pw, double b1, double b2) {
-  ++*step;
-  pw[0] *= b1;
-  pw[1] *= b2;
+// A training minibatch's inputs: dst row b = src row idx[*step * B + b], and
+// dstt = dst^T, in 32 x 32 tiles through shared memory (the step counter lives
+// on the device, so one captured step replays for all).  Columns past `cols`
+// up to ldd are copied too (the GEMM's padded width).
+__global__ void k_gather_inputs(const bf16* __restrict__ src, int64_t lds, const int32_t* __restrict__ idx,
+                                const int* __restrict__ step, int B, int cols, bf16* __restrict__ dst, int64_t ldd,
+                                bf16* __restrict__ dstt, int64_t lddt) {
+  __shared__ bf16 tile[32][33];
+  const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32, c = c0 + threadIdx.x;
+  const int32_t* rows = idx + (int64_t)*step * B;
+  for (int k = threadIdx.y; k < 32; k += blockDim.y) {
+    const int r = r0 + k;
+    if (r < B && c < ldd) {
+      const bf16 v = src[(int64_t)rows[r] * lds + c];
+      dst[(int64_t)r * ldd + c] = v;
+      tile[k][threadIdx.x] = v;
+    }
+  }
+  __syncthreads();
+  for (int k = threadIdx.y; k < 32; k += blockDim.y) {
+    const int ct = c0 + k, r = r0 + threadIdx.x;
+    if (r < B && ct < cols) dstt[(int64_t)ct * lddt + r] = tile[threadIdx.x][k];
+  }
 }
 
 // dst [cols x ldd] = src [rows x cols]^T (BF16), 32 x 32 tiles through shared memory.
@@ -365,17 +354,20 @@ __global__ void k_transpose_bf16(const bf16* __restrict__ src, int64_t lds, int 
 // Output gradient of the mean squared error: dY = 2 (Y - T) / (B d_out) in
 // BF16, row-major and transposed, and per-block float64 partial sums of
 // (Y - T)^2.  32 x 32 tiles; block partials at part[blockIdx.y * gridDim.x + blockIdx.x].
-__global__ void k_loss_dy(const float* __restrict__ Y, int64_t ldy, const float* __restrict__ T, int64_t ldt, int B,
-                          int D, float scale, bf16* __restrict__ dy, int64_t lddy, bf16* __restrict__ dyt,
-                          int64_t lddt, double* __restrict__ part) {
+// Row r's target is row r of T, or row idx[*step * B + r] of it when idx is given.
+__global__ void k_loss_dy(const float* __restrict__ Y, int64_t ldy, const float* __restrict__ T, int64_t ldt,
+                          const int32_t* __restrict__ idx, const int* __restrict__ step, int B, int D, float scale,
+                          bf16* __restrict__ dy, int64_t lddy, bf16* __restrict__ dyt, int64_t lddt,
+                          double* __restrict__ part) {
   __shared__ bf16 tile[32][33];
   __shared__ double red[8];
   const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
+  const int32_t* rows = idx ? idx + (int64_t)*step * B : nullptr;
   float acc = 0.0f;  // a thread's four squares in float32; the block's warps' sums in float64
   for (int k = threadIdx.y; k < 32; k += blockDim.y) {
     const int r = r0 + k, c = c0 + threadIdx.x;
     if (r < B && c < D) {
-      const float d = Y[(int64_t)r * ldy + c] - T[(int64_t)r * ldt + c];
+      const float d = Y[(int64_t)r * ldy + c] - T[(int64_t)(rows ? rows[r] : r) * ldt + c];
       acc = fmaf(d, d, acc);
       const bf16 g = __float2bfloat16_rn(d * scale);
       dy[(int64_t)r * lddy + c] = g;
@@ -397,10 +389,8 @@ __global__ void k_loss_dy(const float* __restrict__ Y, int64_t ldy, const float*
   }
 }
 
-// out[0] = scale * sum of part[0..count) in a fixed order (one block).
-// out[step ? *step : 0] = scale * sum of part[0 .. count)
-__global__ void k_sum_partials(const double* __restrict__ part, int count, double scale, double* __restrict__ out,
-                               const int* __restrict__ step) {
+// out = scale * sum of part[0 .. count) in a fixed order, by one block of 256 threads.
+__device__ __forceinline__ void sum_partials(const double* __restrict__ part, int count, double scale, double* out) {
   __shared__ double red[256];
   double a = 0.0;
   for (int k = threadIdx.x; k < count; k += 256) a += part[k];
@@ -410,17 +400,31 @@ __global__ void k_sum_partials(const double* __restrict__ part, int count, doubl
     if (threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
     __syncthreads();
   }
-  if (threadIdx.x == 0) out[step ? *step : 0] = red[0] * scale;
+  if (threadIdx.x == 0) *out = red[0] * scale;
+}
+
+__global__ void k_sum_partials(const double* __restrict__ part, int count, double scale, double* __restrict__ out) {
+  sum_partials(part, count, scale, out);
+}
+
+// End of a training step (one block): its loss, then the next step's number and beta^t.
+__global__ void k_step_end(const double* __restrict__ part, int count, double scale, double* __restrict__ losses,
+                           int* __restrict__ step, double* __restrict__ pw, double b1, double b2) {
+  sum_partials(part, count, scale, losses + *step);
+  if (threadIdx.x == 0) {  // the thread that has written the loss
+    ++*step;
+    pw[0] *= b1;
+    pw[1] *= b2;
+  }
 }
 
 // out[row] = sum over the first `cols` entries of a BF16 row (one warp per row).
 // One block of 256 threads per row (blockIdx.x): thread t sums columns
 // t, t + 256, ... (pairs of columns when the row start and length allow),
 // then warps and the block reduce in a fixed order.
-__global__ void k_rowsum_bf16(const bf16* __restrict__ src, int64_t lds, int rows, int cols, float* __restrict__ out) {
+// Returns the sum on thread 0.
+__device__ __forceinline__ float row_sum_bf16(const bf16* __restrict__ src, int64_t lds, int r, int cols) {
   __shared__ float wsum[8];
-  const int r = blockIdx.x;
-  if (r >= rows) return;
   const bf16* row = src + (int64_t)r * lds;
   float a = 0.0f;
   if ((lds & 1) == 0 && (cols & 1) == 0 && (reinterpret_cast<uintptr_t>(src) & 3) == 0) {
@@ -436,11 +440,17 @@ __global__ void k_rowsum_bf16(const bf16* __restrict__ src, int64_t lds, int row
   for (int off = 16; off > 0; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
   if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = a;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    float t = 0.0f;
+  float t = 0.0f;
+  if (threadIdx.x == 0)
     for (int w = 0; w < 8; ++w) t += wsum[w];
-    out[r] = t;
-  }
+  return t;
+}
+
+__global__ void k_rowsum_bf16(const bf16* __restrict__ src, int64_t lds, int rows, int cols, float* __restrict__ out) {
+  const int r = blockIdx.x;
+  if (r >= rows) return;
+  const float t = row_sum_bf16(src, lds, r, cols);
+  if (threadIdx.x == 0) out[r] = t;
 }
 
 // out[k] = sum_s P[s * stride + k], s ascending.
@@ -457,22 +467,92 @@ __global__ void k_sum_slices(const float* __restrict__ P, int S, int64_t stride,
 // Adam (Kingma and Ba 2015, Algorithm 1) on the float32 master parameters.
 // Adam with the bias corrections bc1, bc2, or 1 - pw[0], 1 - pw[1] when pw
 // (this step's beta1^t, beta2^t, kept on the device) is given.
-__global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m, float* __restrict__ v,
-                       int64_t count, float lr, float b1, float b2, float eps, float bc1, float bc2,
-                       const double* __restrict__ pw) {
-  const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (k >= count) return;
-  if (pw) {
-    bc1 = (float)(1.0 - pw[0]);
-    bc2 = (float)(1.0 - pw[1]);
-  }
-  const float gk = g[k];
-  const float mk = b1 * m[k] + (1.0f - b1) * gk;
-  const float vk = b2 * v[k] + (1.0f - b2) * gk * gk;
-  m[k] = mk;
-  v[k] = vk;
+struct AdamArgs {
+  float *p, *m, *v;
+  float lr, b1, b2, eps;
+};
+__device__ __forceinline__ float adam_update(const AdamArgs& a, int64_t k, float gk, float bc1, float bc2) {
+  const float mk = a.b1 * a.m[k] + (1.0f - a.b1) * gk;
+  const float vk = a.b2 * a.v[k] + (1.0f - a.b2) * gk * gk;
+  a.m[k] = mk;
+  a.v[k] = vk;
   const float mh = mk / bc1, vh = vk / bc2;
-  p[k] -= lr * mh / (sqrtf(vh) + eps);
+  const float pk = a.p[k] - a.lr * mh / (sqrtf(vh) + a.eps);
+  a.p[k] = pk;
+  return pk;
+}
+
+__global__ void k_adam(AdamArgs a, const float* __restrict__ g, int64_t count, float bc1, float bc2) {
+  const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (k < count) adam_update(a, k, g[k], bc1, bc2);
+}
+
+// The whole update of a training step in one launch: every parameter's
+// gradient from what the backward pass left behind, Adam, and the BF16 copies.
+// Blocks [wblk[l], wblk[l + 1]) take 32 x 32 tiles of W_l, whose split-K slices
+// they sum (ascending); the blocks after them one bias each, the sum of a row
+// of dZ_l^T.  As four launches a layer and six more, at 4-6 us each, this took
+// 62 us of a 236 us step (network 258-3x256-576, batch 8 192).
+constexpr int kUpdMaxLayers = 8;  // layers of one launch (deeper networks take several)
+struct UpdateArgs {
+  int L, B;
+  int64_t ldB;
+  int N[kUpdMaxLayers], K[kUpdMaxLayers], S[kUpdMaxLayers], tiles_k[kUpdMaxLayers];
+  int wblk[kUpdMaxLayers + 1], bblk[kUpdMaxLayers + 1];
+  const float* slices[kUpdMaxLayers];
+  const bf16* dzt[kUpdMaxLayers];
+  int64_t off_w[kUpdMaxLayers], off_b[kUpdMaxLayers];
+  bf16 *w16[kUpdMaxLayers], *wt16[kUpdMaxLayers];
+  int ldk[kUpdMaxLayers], ldn[kUpdMaxLayers];
+};
+
+__global__ void __launch_bounds__(256) k_train_update(const __grid_constant__ UpdateArgs u, const AdamArgs a,
+                                                      const double* __restrict__ pw) {
+  const int blk = blockIdx.x;
+  const float bc1 = (float)(1.0 - pw[0]), bc2 = (float)(1.0 - pw[1]);
+  if (blk >= u.wblk[u.L]) {
+    int l = 0;
+    while (blk >= u.bblk[l + 1]) ++l;
+    const int n = blk - u.bblk[l];
+    const float g = row_sum_bf16(u.dzt[l], u.ldB, n, u.B);
+    if (threadIdx.x == 0) adam_update(a, u.off_b[l] + n, g, bc1, bc2);
+    return;
+  }
+  int l = 0;
+  while (blk >= u.wblk[l + 1]) ++l;
+  const int N = u.N[l], K = u.K[l], S = u.S[l], t = blk - u.wblk[l];
+  const int n0 = (t / u.tiles_k[l]) * 32, k0 = (t % u.tiles_k[l]) * 32;
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const int64_t stride = (int64_t)N * K;
+  const float* P = u.slices[l];
+  __shared__ bf16 tile[32][33];
+  float g[4] = {0.f, 0.f, 0.f, 0.f};
+  const int k = k0 + tx;
+  if (k < K) {
+#pragma unroll 8
+    for (int s = 0; s < S; ++s) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int n = n0 + ty + 8 * q;
+        if (n < N) g[q] += P[s * stride + (int64_t)n * K + k];
+      }
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int n = n0 + ty + 8 * q;
+    if (n < N && k < K) {
+      const bf16 w = __float2bfloat16_rn(adam_update(a, u.off_w[l] + (int64_t)n * K + k, g[q], bc1, bc2));
+      u.w16[l][(int64_t)n * u.ldk[l] + k] = w;
+      tile[ty + 8 * q][tx] = w;
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int kk = k0 + ty + 8 * q, n = n0 + tx;
+    if (n < N && kk < K) u.wt16[l][(int64_t)kk * u.ldn[l] + n] = tile[tx][ty + 8 * q];
+  }
 }
 
 // BF16 copies of one weight matrix W [N x K]: W16 [N x ldk], W16^T [K x ldn].
@@ -493,6 +573,13 @@ unsigned blocks_for(int64_t count, int threads) { return (unsigned)((count + thr
 // ---------------------------------------------------------------------------
 // The network
 // ---------------------------------------------------------------------------
+// What a layer's gradients are summed from after the backward pass.
+struct LayerGrad {
+  int N, K, S;          // W is [N x K], in S slices of N K values
+  const float* slices;
+  const bf16* dzt;      // [N x ldB] dZ^T
+};
+
 struct MlpNet {
   std::vector<int> dims;           // d_in, hidden..., d_out
   int L = 0;                       // layers (hidden + output)
@@ -506,10 +593,11 @@ struct MlpNet {
   std::vector<DBuf<float>> z32;    // [B x N_l] pre-activations of hidden layers
   std::vector<DBuf<bf16>> h16, ht16;
   DBuf<float> y32;
-  DBuf<bf16> dy16, dyt16, dz16[2], dzt16[2];
-  DBuf<float> partial;
+  DBuf<bf16> dy16, dyt16, dz16[2];
+  std::vector<DBuf<bf16>> dzt16;   // [N_l x ldB] transposed pre-activation gradients of hidden layers
+  DBuf<float> partial;             // split-K slices of the layers' weight gradients, layer l at off_part[l]
+  std::vector<int64_t> off_part;   // [L + 1]; a layer without room here is not split and goes to `grad`
   DBuf<bf16> xb, xbt;
-  DBuf<float> tb;
   DBuf<double> loss_part, loss_hist;
   DBuf<int> step_dev;  // training step within a cc_mlp_train call
   DBuf<double> adam_pw;     // that step's beta1^t, beta2^t
@@ -565,40 +653,36 @@ struct MlpNet {
     }
   }
 
-  // Loss into loss_dev[step ? *step : 0], gradient into `grad` (all
-  // parameters).  xbt holds X^T.
-  void backward(const float* T, int64_t ldt, int B, double* loss_dev, const int* step = nullptr) {
+  // Gradient of the loss: what the parameters' gradients are summed from stays
+  // in `partial` or `grad` (weights) and dzt16 / dyt16 (biases, rows), as `out`
+  // says.  Targets are rows 0 .. B - 1 of T, or those of idx at *step.
+  // xbt holds X^T; the loss's block partials go to loss_part.
+  void backward(const float* T, int64_t ldt, const int32_t* idx, const int* step, int B,
+                std::vector<LayerGrad>& out) {
     const int D = d_out();
-    {
-      const dim3 grid((unsigned)((D + 31) / 32), (unsigned)((B + 31) / 32));
-      k_loss_dy<<<grid, dim3(32, 8), 0, stream>>>(y32.p, D, T, ldt, B, D, 2.0f / ((float)B * (float)D), dy16.p, D,
-                                                  dyt16.p, ldB, loss_part.p);
-      CCG_CUDA(cudaGetLastError());
-      k_sum_partials<<<1, 256, 0, stream>>>(loss_part.p, (int)(grid.x * grid.y), 1.0 / ((double)B * D), loss_dev,
-                                            step);
-      CCG_CUDA(cudaGetLastError());
-    }
+    const dim3 grid = loss_grid(B);
+    k_loss_dy<<<grid, dim3(32, 8), 0, stream>>>(y32.p, D, T, ldt, idx, step, B, D, 2.0f / ((float)B * (float)D), dy16.p,
+                                                D, dyt16.p, ldB, loss_part.p);
+    CCG_CUDA(cudaGetLastError());
+    out.resize(L);
     const bf16* dz = dy16.p;
-    const bf16* dzt = dyt16.p;
     int cur = 0;
     for (int l = L - 1; l >= 0; --l) {
       const int N = dims[l + 1], K = dims[l];
+      const bf16* dzt = l == L - 1 ? dyt16.p : dzt16[l].p;
       // weight gradient dW_l = dZ^T H_{l-1}: [N x K], contraction over the batch
       const bf16* Ht = l == 0 ? xbt.p : ht16[l - 1].p;
       const GemmShape sh = gemm_pick_shape(N, K, B, true);
       GemmEpilogue ep;
-      ep.c32 = partial.p;
+      const int64_t room = off_part[l + 1] - off_part[l];
+      ep.c32 = room > 0 ? partial.p + off_part[l] : grad.p + off_w[l];
       ep.ldc = K;
       ep.split_stride = (int64_t)N * K;
-      CCG_CHECK((int64_t)sh.splits * N * K <= (int64_t)partial.count, CC_ERR_STATE, "split-K workspace too small");
+      CCG_CHECK((int64_t)sh.splits * N * K <= (room > 0 ? room : (int64_t)N * K), CC_ERR_STATE,
+                "split-K workspace too small");
       gemm_tn(dzt, ldB, Ht, ldB, N, K, B, kEpiF32, ep, err.p, stream, sh);
-      const int kt = (B + 63) / 64, per = (kt + sh.splits - 1) / sh.splits, S = (kt + per - 1) / per;
-      k_sum_slices<<<blocks_for((int64_t)N * K, 256), 256, 0, stream>>>(partial.p, S, (int64_t)N * K, (int64_t)N * K,
-                                                                        grad.p + off_w[l], K, K, K);
-      CCG_CUDA(cudaGetLastError());
-      // bias gradient: row sums of dZ^T
-      k_rowsum_bf16<<<(unsigned)N, 256, 0, stream>>>(dzt, ldB, N, B, grad.p + off_b[l]);
-      CCG_CUDA(cudaGetLastError());
+      const int kt = (B + 63) / 64, per = (kt + sh.splits - 1) / sh.splits;
+      out[l] = LayerGrad{N, K, (kt + per - 1) / per, ep.c32, dzt};
       if (l == 0) break;
       // input gradient dH_{l-1} = dZ W_l, times gelu'(Z_{l-1}) in the epilogue
       GemmEpilogue eg;
@@ -606,12 +690,71 @@ struct MlpNet {
       eg.ldz = K;
       eg.h16 = dz16[cur].p;
       eg.ldh = K;
-      eg.ht16 = dzt16[cur].p;
+      eg.ht16 = dzt16[l - 1].p;
       eg.ldt = ldB;
       gemm_tn(dz, N, wt16[l].p, ldn[l], B, K, N, kEpiGeluGrad, eg, err.p, stream, gemm_pick_shape(B, K, N, false));
       dz = dz16[cur].p;
-      dzt = dzt16[cur].p;
       cur ^= 1;
+    }
+  }
+
+  dim3 loss_grid(int B) const { return dim3((unsigned)((d_out() + 31) / 32), (unsigned)((B + 31) / 32)); }
+
+  // loss into loss_hist[0], gradient of rows 0 .. B - 1 into `grad`
+  void loss_grad(const float* T, int64_t ldt, int B) {
+    std::vector<LayerGrad> lg;
+    backward(T, ldt, nullptr, nullptr, B, lg);
+    const dim3 grid = loss_grid(B);
+    k_sum_partials<<<1, 256, 0, stream>>>(loss_part.p, (int)(grid.x * grid.y), 1.0 / ((double)B * d_out()),
+                                          loss_hist.p);
+    CCG_CUDA(cudaGetLastError());
+    for (int l = L - 1; l >= 0; --l) {
+      const LayerGrad& d = lg[l];
+      const int64_t count = (int64_t)d.N * d.K;
+      if (d.slices != grad.p + off_w[l]) {
+        k_sum_slices<<<blocks_for(count, 256), 256, 0, stream>>>(d.slices, d.S, count, count, grad.p + off_w[l], d.K,
+                                                                 d.K, d.K);
+        CCG_CUDA(cudaGetLastError());
+      }
+      k_rowsum_bf16<<<(unsigned)d.N, 256, 0, stream>>>(d.dzt, ldB, d.N, B, grad.p + off_b[l]);
+      CCG_CUDA(cudaGetLastError());
+    }
+  }
+
+  // parameters, Adam's moments and the BF16 weights after backward()
+  void train_update(const std::vector<LayerGrad>& lg, int B, const cc_adam& o) {
+    for (int l0 = 0; l0 < L; l0 += kUpdMaxLayers) {
+      UpdateArgs u;
+      u.L = std::min(kUpdMaxLayers, L - l0);
+      u.B = B;
+      u.ldB = ldB;
+      int at = 0;
+      for (int k = 0; k < u.L; ++k) {
+        const LayerGrad& d = lg[l0 + k];
+        u.N[k] = d.N;
+        u.K[k] = d.K;
+        u.S[k] = d.S;
+        u.slices[k] = d.slices;
+        u.dzt[k] = d.dzt;
+        u.wblk[k] = at;
+        u.tiles_k[k] = (d.K + 31) / 32;
+        at += u.tiles_k[k] * ((d.N + 31) / 32);
+        u.off_w[k] = off_w[l0 + k];
+        u.off_b[k] = off_b[l0 + k];
+        u.w16[k] = w16[l0 + k].p;
+        u.wt16[k] = wt16[l0 + k].p;
+        u.ldk[k] = ldk[l0 + k];
+        u.ldn[k] = ldn[l0 + k];
+      }
+      u.wblk[u.L] = at;
+      for (int k = 0; k < u.L; ++k) {
+        u.bblk[k] = at;
+        at += lg[l0 + k].N;
+      }
+      u.bblk[u.L] = at;
+      k_train_update<<<(unsigned)at, 256, 0, stream>>>(
+          u, AdamArgs{params.p, adam_m.p, adam_v.p, o.lr, o.beta1, o.beta2, o.eps}, adam_pw.p);
+      CCG_CUDA(cudaGetLastError());
     }
   }
 
@@ -619,16 +762,8 @@ struct MlpNet {
     ++adam_t;
     const double bc1 = 1.0 - std::pow((double)o.beta1, (double)adam_t);
     const double bc2 = 1.0 - std::pow((double)o.beta2, (double)adam_t);
-    k_adam<<<blocks_for(nparams, 256), 256, 0, stream>>>(params.p, g, adam_m.p, adam_v.p, nparams, o.lr, o.beta1,
-                                                         o.beta2, o.eps, (float)bc1, (float)bc2, nullptr);
-    CCG_CUDA(cudaGetLastError());
-    refresh_bf16();
-  }
-
-  // Adam with this step's beta^t from the device (the training loop)
-  void adam_dev(const float* g, const cc_adam& o) {
-    k_adam<<<blocks_for(nparams, 256), 256, 0, stream>>>(params.p, g, adam_m.p, adam_v.p, nparams, o.lr, o.beta1,
-                                                         o.beta2, o.eps, 1.0f, 1.0f, adam_pw.p);
+    k_adam<<<blocks_for(nparams, 256), 256, 0, stream>>>(
+        AdamArgs{params.p, adam_m.p, adam_v.p, o.lr, o.beta1, o.beta2, o.eps}, g, nparams, (float)bc1, (float)bc2);
     CCG_CUDA(cudaGetLastError());
     refresh_bf16();
   }
@@ -824,7 +959,7 @@ cc_status cc_mlp_create(const cc_mlp_config* cfg, void* stream, cc_mlp** out) {
     CCG_CUDA(cudaMemsetAsync(net->adam_v.p, 0, o * sizeof(float), s));
     net->w16.resize(net->L);
     net->wt16.resize(net->L);
-    int64_t part = 1;
+    net->off_part.assign(1, 0);
     for (int l = 0; l < net->L; ++l) {
       const int N = net->dims[l + 1], K = net->dims[l];
       net->w16[l].alloc((size_t)N * net->ldk[l]);
@@ -832,7 +967,8 @@ cc_status cc_mlp_create(const cc_mlp_config* cfg, void* stream, cc_mlp** out) {
       CCG_CUDA(cudaMemsetAsync(net->w16[l].p, 0, (size_t)N * net->ldk[l] * sizeof(bf16), s));
       CCG_CUDA(cudaMemsetAsync(net->wt16[l].p, 0, (size_t)K * net->ldn[l] * sizeof(bf16), s));
       const GemmShape sh = gemm_pick_shape(N, K, net->max_batch, true);
-      part = std::max<int64_t>(part, (int64_t)sh.splits * N * K);
+      // 16-byte aligned starts
+      net->off_part.push_back(net->off_part.back() + (sh.splits > 1 ? ((int64_t)sh.splits * N * K + 3) / 4 * 4 : 0));
     }
     const int B = net->max_batch, ldB = net->ldB;
     net->z32.resize(net->L - 1);
@@ -849,14 +985,12 @@ cc_status cc_mlp_create(const cc_mlp_config* cfg, void* stream, cc_mlp** out) {
     net->y32.alloc((size_t)B * cfg->d_out);
     net->dy16.alloc((size_t)B * cfg->d_out);
     net->dyt16.alloc((size_t)cfg->d_out * ldB);
-    for (int c = 0; c < 2; ++c) {
-      net->dz16[c].alloc((size_t)B * hmax);
-      net->dzt16[c].alloc((size_t)hmax * ldB);
-    }
-    net->partial.alloc((size_t)part);
+    for (int c = 0; c < 2; ++c) net->dz16[c].alloc((size_t)B * hmax);
+    net->dzt16.resize(net->L - 1);
+    for (int l = 0; l + 1 < net->L; ++l) net->dzt16[l].alloc((size_t)net->dims[l + 1] * ldB);
+    net->partial.alloc((size_t)net->off_part.back());
     net->xb.alloc((size_t)B * round8(cfg->d_in));
     net->xbt.alloc((size_t)cfg->d_in * ldB);
-    net->tb.alloc((size_t)B * cfg->d_out);
     net->loss_part.alloc((size_t)((cfg->d_out + 31) / 32) * ((B + 31) / 32));
     net->loss_hist.alloc(1);
     net->step_dev.alloc(1);
@@ -988,7 +1122,7 @@ cc_status cc_mlp_loss_grad(cc_mlp* net, const void* X, int64_t ldx, const float*
     const bf16* Xb = static_cast<const bf16*>(X);
     net->transpose_input(Xb, ldx, rows);
     net->forward_train(Xb, ldx, rows);
-    net->backward(T, ldt, rows, net->loss_hist.p);
+    net->loss_grad(T, ldt, rows);
     if (grad) CCG_CUDA(cudaMemcpyAsync(grad, net->grad.p, net->nparams * sizeof(float), cudaMemcpyDeviceToDevice, s));
     double h = 0.0;
     CCG_CUDA(cudaMemcpyAsync(&h, net->loss_hist.p, sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -1018,12 +1152,9 @@ cc_status cc_mlp_train(cc_mlp* net, const void* X, int64_t ldx, const float* T, 
     if (steps == 0) return CC_OK;
     net->loss_hist.alloc(steps);
     const int ldxb = round8(net->d_in());
-    const int chunks = ldxb / 8;
     const int64_t t0 = net->adam_t;
     int* step = net->step_dev.p;
     CCG_CUDA(cudaMemsetAsync(step, 0, sizeof(int), s));
-    const bool vec4 = net->d_out() % 4 == 0 && ldt % 4 == 0 && (reinterpret_cast<uintptr_t>(T) & 15) == 0 &&
-                      (reinterpret_cast<uintptr_t>(net->tb.p) & 15) == 0;
     // beta^t of the first step; each step's advance multiplies them by beta
     net->adam_pw_host[0] = std::pow((double)opt->beta1, (double)(t0 + 1));
     net->adam_pw_host[1] = std::pow((double)opt->beta2, (double)(t0 + 1));
@@ -1032,25 +1163,20 @@ cc_status cc_mlp_train(cc_mlp* net, const void* X, int64_t ldx, const float* T, 
     // from the device step counter, which the step advances last
     auto one_step = [&]() {
       cudaStream_t q = net->stream;
-      k_gather_rows_bf16<<<blocks_for((int64_t)batch * chunks, 256), 256, 0, q>>>(
-          static_cast<const bf16*>(X), ldx, idx, step, batch, chunks, net->xb.p, ldxb);
+      k_gather_inputs<<<dim3((unsigned)((ldxb + 31) / 32), (unsigned)((batch + 31) / 32)), dim3(32, 8), 0, q>>>(
+          static_cast<const bf16*>(X), ldx, idx, step, batch, net->d_in(), net->xb.p, ldxb, net->xbt.p, net->ldB);
       CCG_CUDA(cudaGetLastError());
-      if (vec4)
-        k_gather_rows_f32<4><<<blocks_for((int64_t)batch * net->d_out() / 4, 256), 256, 0, q>>>(
-            T, ldt, idx, step, batch, net->d_out(), net->tb.p, net->d_out());
-      else
-        k_gather_rows_f32<1><<<blocks_for((int64_t)batch * net->d_out(), 256), 256, 0, q>>>(
-            T, ldt, idx, step, batch, net->d_out(), net->tb.p, net->d_out());
-      CCG_CUDA(cudaGetLastError());
-      net->transpose_input(net->xb.p, ldxb, batch);
       net->forward_train(net->xb.p, ldxb, batch);
-      net->backward(net->tb.p, net->d_out(), batch, net->loss_hist.p, step);
-      net->adam_dev(net->grad.p, *opt);
-      k_step_advance<<<1, 1, 0, q>>>(step, net->adam_pw.p, (double)opt->beta1, (double)opt->beta2);
+      std::vector<LayerGrad> lgr;
+      net->backward(T, ldt, idx, step, batch, lgr);
+      net->train_update(lgr, batch, *opt);
+      const dim3 lg = net->loss_grid(batch);
+      k_step_end<<<1, 256, 0, q>>>(net->loss_part.p, (int)(lg.x * lg.y), 1.0 / ((double)batch * net->d_out()),
+                                   net->loss_hist.p, step, net->adam_pw.p, (double)opt->beta1, (double)opt->beta2);
       CCG_CUDA(cudaGetLastError());
     };
     // the first step runs directly (it also fills every host-side cache the
-    // launches use); the others replay one captured step (about 30 launches).
+    // launches use); the others replay one captured step (15 launches for four layers).
     // The legacy default stream cannot be captured: the step is then recorded
     // on a private stream, and the graph still runs on the network's stream.
     one_step();

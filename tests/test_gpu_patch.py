@@ -31,12 +31,10 @@ def test_every_patch_size_matches_the_oracle():
     size = np.diff(ptr)
     free = np.flatnonzero(size)
     sup = [idx[ptr[v]:ptr[v + 1]] for v in range(sc.n)]
-    for q, v in enumerate(free):  # every second vertex takes the next size, nearest vertices first
-        if q % 2 == 0:
-            near = np.argsort(np.linalg.norm(sc.X[sup[v]] - sc.X[v], axis=1), kind="stable")[:1 + (q // 2) % 64]
-            sup[v] = np.sort(sup[v][near])
-    seen = {s.size for s in sup}
-    assert max(seen) == 64 and len(seen & set(range(1, 65))) >= 60
+    for q, v in enumerate(free[np.argsort(-size[free], kind="stable")][:64]):  # sizes 64, 63, .., 1, nearest first
+        near = np.argsort(np.linalg.norm(sc.X[sup[v]] - sc.X[v], axis=1), kind="stable")[:64 - q]
+        sup[v] = np.sort(sup[v][near])
+    assert set(range(1, 65)) <= {s.size for s in sup}
     m.set_subspace(np.concatenate([[0], np.cumsum([s.size for s in sup])]), np.concatenate(sup),
                    np.zeros((sum(s.size for s in sup), 3, 3)))
     assert m.build_subspace_at(cc.to_soa(x)) == 0
