@@ -91,6 +91,8 @@ void ensure_state(Mesh& m, cc_precision p) {
     }
     if (rows_from_positions(m, true)) {
       if (!m.mx.rec.p) {
+        m.mx.diag_g.alloc(3 * m.n);
+        CCG_CUDA(cudaMemsetAsync(m.mx.diag_g.p, 0, 3 * m.n * sizeof(float4), s));
         m.mx.rec.alloc(m.T);
         CCG_CUDA(cudaMemsetAsync(m.mx.rec.p, 0, m.T * sizeof(float4), s));
       }

@@ -96,6 +96,14 @@ constexpr int kTetStore = 80;
 // copies a vertex's map in 4-byte words from the word holding its first code,
 // which reads up to 3 codes past the map's end.
 constexpr int kSlotMapSlack = 8;
+// Where row r of upper block q of a block row lies (in values): the row has
+// `len` blocks from block p0 on.  Float64 blocks are 3 x 4 each, one after the
+// other; a float32 block row is three planes, plane r the r-th rows of all its
+// blocks, so that lanes taking neighbouring blocks read neighbouring 16 bytes.
+template <typename HT>
+__host__ __device__ constexpr int64_t block_row_at(int64_t p0, int len, int q, int r) {
+  return sizeof(HT) == 4 ? 12 * p0 + 4 * ((int64_t)r * len + q) : 12 * (p0 + q) + 4 * r;
+}
 // Fields of a pair-list entry (Mesh::d_pairs).
 constexpr int kPairMaxSup = 1020, kPairMaxRow = 4095;
 constexpr uint32_t kPairSelf = 1023;
@@ -126,7 +134,8 @@ struct StateMixed {
   DBuf<float4> rec;   // [T] (sigma hi, sigma lo, c1, 0) of every tet (rows formed from the positions)
   DBuf<float> g_hi;   // [n][3]
   DBuf<float> g_lo;   // [n][3]
-  DBuf<float> bsr;    // [nnz_up][12]
+  DBuf<float> bsr;    // [nnz_up][12], a row in three planes (block_row_at)
+  DBuf<float4> diag_g;  // [n][3] (H_jj 00 01 02 11 12 22, g) of rows formed from the positions
   DBuf<float> U;      // [sup_total][9]
   DBuf<float> cpl;    // [n_free][32]
   DBuf<float> rot;    // [n][9] per-vertex rotations of corotated bases
@@ -262,8 +271,8 @@ struct Mesh {
   // |S_i|, and kPairSelf as column slot marks a block (j, i) of a support row.
   // Empty when a support or a row does not fit the fields.
   bool pairs_ok = false;
-  DBuf<int4> d_pair_hdr;       // [2n] (first support entry, |S_i|, pairs, ns), (list start lo, hi, first block of row i, 0)
-  DBuf<int32_t> d_sup_row;     // [support_total] first upper block of every support vertex's row
+  DBuf<int4> d_pair_hdr;       // [2n] (first support entry, |S_i|, pairs, ns), (list start lo, hi, first block of row i, blocks)
+  DBuf<int2> d_sup_row;        // [support_total] first upper block and blocks of every support vertex's row
   DBuf<uint32_t> d_pairs;
   // rows formed from the positions (kernels_rows.cu; stable Neo-Hookean)
   bool rows_ok = false;      // the mesh fits that kernel (build_row_data)

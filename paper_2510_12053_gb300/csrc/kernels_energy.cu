@@ -483,7 +483,7 @@ __global__ void k_row_gather(const int4* __restrict__ row_hdr, int64_t nrows, co
     if (lane < 9) {
       HT d = (acc + a1) + a2;
       if (dynamic && r == col) d += massh[j];
-      HT* dst = bsr + (int64_t)p0 * 12 + 4 * r;
+      HT* dst = bsr + block_row_at<HT>(p0, nup, 0, r);
       dst[col] = d;
       if (col == 2) dst[3] = HT(0);
     }
@@ -499,7 +499,7 @@ __global__ void k_row_gather(const int4* __restrict__ row_hdr, int64_t nrows, co
         const int v = rsrc[s];
         acc += hten[(v & 0x7fffffff) + (v < 0 ? tidx : c)];
       }
-      HT* dst = bsr + (int64_t)(p0 + q) * 12 + 4 * r;
+      HT* dst = bsr + block_row_at<HT>(p0, nup, q, r);
       dst[col] = acc;
       if (col == 2) dst[3] = HT(0);
     }

@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(256, 3) k_rows_mixed(
     const int32_t* __restrict__ rs_ptr, const uint16_t* __restrict__ rs_code, const float4* __restrict__ x_hi,
     const float4* __restrict__ x_lo, float scale, float inv_scale, const float2* __restrict__ mass_df,
     const float4* __restrict__ xt_hi, const float4* __restrict__ xt_lo, bool dynamic, int max_val, int max_ring,
-    float* __restrict__ bsr, float* __restrict__ g_hi, float* __restrict__ g_lo) {
+    float* __restrict__ bsr, float* __restrict__ g_hi, float* __restrict__ g_lo, float4* __restrict__ diag_g) {
   pdl_entry();
   extern __shared__ __align__(16) float4 rows_smem[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sub = lane >> 3, t = lane & 7;
@@ -265,11 +265,17 @@ __global__ void __launch_bounds__(256, 3) k_rows_mixed(
     g_lo[3 * (int64_t)j + t] = g.lo;
   }
   for (int q = t; q < nup; q += 8) {
-    float4* dst = reinterpret_cast<float4*>(bsr + (int64_t)(q0 + q) * 12);
+    float4* dst = reinterpret_cast<float4*>(bsr) + block_row_at<float>(q0, nup, q, 0) / 4;
     if (q == 0) {
       dst[0] = make_float4(dg[0] + mq, dg[1], dg[2], 0.f);
-      dst[1] = make_float4(dg[1], dg[3] + mq, dg[4], 0.f);
-      dst[2] = make_float4(dg[2], dg[4], dg[5] + mq, 0.f);
+      dst[nup] = make_float4(dg[1], dg[3] + mq, dg[4], 0.f);
+      dst[2 * nup] = make_float4(dg[2], dg[4], dg[5] + mq, 0.f);
+      if (!dynamic) {
+        float4* own = diag_g + 3 * (int64_t)j;
+        own[0] = make_float4(dg[0] + mq, dg[1], dg[2], dg[3] + mq);
+        own[1] = make_float4(dg[4], dg[5] + mq, gd[0].hi * inv_scale, gd[1].hi * inv_scale);
+        own[2] = make_float4(gd[2].hi * inv_scale, 0.f, 0.f, 0.f);
+      }
       continue;
     }
     if (q >= 8) {
@@ -295,8 +301,8 @@ __global__ void __launch_bounds__(256, 3) k_rows_mixed(
         for (int c = 0; c < 3; ++c) H[3 * rr + c] = fmaf(n0[rr], nk[c], H[3 * rr + c]);
     });
     dst[0] = make_float4(H[0], H[1] + y2, H[2] - y1, 0.f);
-    dst[1] = make_float4(H[3] - y2, H[4], H[5] + y0, 0.f);
-    dst[2] = make_float4(H[6] + y1, H[7] - y0, H[8], 0.f);
+    dst[nup] = make_float4(H[3] - y2, H[4], H[5] + y0, 0.f);
+    dst[2 * nup] = make_float4(H[6] + y1, H[7] - y0, H[8], 0.f);
   }
 }
 
@@ -560,7 +566,7 @@ void launch_rows_from_positions(Mesh& m, bool mixed, const double* x, const doub
                (const uint4*)m.d_codes8.p, (const int32_t*)m.d_rs_ptr.p, (const uint16_t*)m.d_rs_code.p,
                (const float4*)m.mx.x_hi.p, (const float4*)m.mx.x_lo.p, m.len_scale, 1.0f / m.len_scale,
                (const float2*)m.d_mass_df.p, (const float4*)m.mx.xt_hi.p, (const float4*)m.mx.xt_lo.p, dyn,
-               (int)m.max_valence, (int)m.max_ring, m.mx.bsr.p, m.mx.g_hi.p, m.mx.g_lo.p);
+               (int)m.max_valence, (int)m.max_ring, m.mx.bsr.p, m.mx.g_hi.p, m.mx.g_lo.p, m.mx.diag_g.p);
   } else {
     set_smem_limit(reinterpret_cast<const void*>(k_rows_f64), wpb * per);
     pdl_launch(k_rows_f64, grid, 32 * wpb, wpb * per, s, (const int4*)m.d_row_hdr2.p, m.n_free,

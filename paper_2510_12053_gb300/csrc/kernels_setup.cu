@@ -313,7 +313,7 @@ template <bool kFill>
 __global__ void k_pair_lists(const int32_t* __restrict__ rows, int64_t nrows, const int32_t* __restrict__ sup_ptr,
                              const int32_t* __restrict__ sup_idx, const int32_t* __restrict__ up_ptr,
                              const int32_t* __restrict__ up_col, int2* __restrict__ counts,
-                             const int4* __restrict__ hdr, int32_t* __restrict__ sup_row,
+                             const int4* __restrict__ hdr, int2* __restrict__ sup_row,
                              uint32_t* __restrict__ list) {
   const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
@@ -335,7 +335,7 @@ __global__ void k_pair_lists(const int32_t* __restrict__ rows, int64_t nrows, co
       const int j = r < m ? S[r] : v;
       p0 = up_ptr[j];
       len = up_ptr[j + 1] - p0;
-      if (kFill && r < m) sup_row[s0 + r] = p0;
+      if (kFill && r < m) sup_row[s0 + r] = make_int2(p0, len);
     }
     // what one block of the lane's row is: 1 a pair, 2 a block with v, 0 neither
     auto kind = [&](int q, uint32_t* col) {
@@ -401,7 +401,8 @@ static void build_pair_lists(Mesh& m) {
     if (m.pinned[v]) continue;
     const int2 c = counts[w++];
     hdr[2 * v] = make_int4((int)m.sup_ptr[v], (int)(m.sup_ptr[v + 1] - m.sup_ptr[v]), c.x, c.y);
-    hdr[2 * v + 1] = make_int4((int)(uint32_t)(at & 0xffffffff), (int)(at >> 32), (int)m.up_ptr[v], 0);
+    hdr[2 * v + 1] = make_int4((int)(uint32_t)(at & 0xffffffff), (int)(at >> 32), (int)m.up_ptr[v],
+                             (int)(m.up_ptr[v + 1] - m.up_ptr[v]));
     at += c.x + c.y;
   }
   m.d_pair_hdr.upload(hdr, s);

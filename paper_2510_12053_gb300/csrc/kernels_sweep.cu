@@ -36,22 +36,23 @@ __device__ __forceinline__ T warp_sum(T v) {
   return v;
 }
 
-// Loads the 3x3 block p of the padded upper rows.
+// Loads upper block q of the block row of len blocks that starts at block p0.
 template <typename HT>
-__device__ __forceinline__ void load_block(const HT* __restrict__ bsr, int64_t p, HT* H);
+__device__ __forceinline__ void load_block(const HT* __restrict__ bsr, int64_t p0, int len, int q, HT* H);
 
 template <>
-__device__ __forceinline__ void load_block<float>(const float* __restrict__ bsr, int64_t p, float* H) {
-  const float4* b = reinterpret_cast<const float4*>(bsr + p * 12);
-  const float4 r0 = __ldg(b), r1 = __ldg(b + 1), r2 = __ldg(b + 2);
+__device__ __forceinline__ void load_block<float>(const float* __restrict__ bsr, int64_t p0, int len, int q, float* H) {
+  const float4* b = reinterpret_cast<const float4*>(bsr) + block_row_at<float>(p0, len, q, 0) / 4;
+  const float4 r0 = __ldg(b), r1 = __ldg(b + len), r2 = __ldg(b + 2 * len);
   H[0] = r0.x; H[1] = r0.y; H[2] = r0.z;
   H[3] = r1.x; H[4] = r1.y; H[5] = r1.z;
   H[6] = r2.x; H[7] = r2.y; H[8] = r2.z;
 }
 
 template <>
-__device__ __forceinline__ void load_block<double>(const double* __restrict__ bsr, int64_t p, double* H) {
-  const double2* b = reinterpret_cast<const double2*>(bsr + p * 12);
+__device__ __forceinline__ void load_block<double>(const double* __restrict__ bsr, int64_t p0, int len, int q,
+                                                   double* H) {
+  const double2* b = reinterpret_cast<const double2*>(bsr + block_row_at<double>(p0, len, q, 0));
 #pragma unroll
   for (int r = 0; r < 3; ++r) {
     const double2 u = __ldg(b + 2 * r), v = __ldg(b + 2 * r + 1);
@@ -190,7 +191,7 @@ __device__ __forceinline__ void condense_vertex(const CondenseArgs<HT>& c, int64
   V H[9], gi[3];
   if (kUpd == CC_UPDATE_CD) {
     HT Hb[9];
-    load_block(c.bsr, c.up_ptr[i], Hb);
+    load_block(c.bsr, c.up_ptr[i], c.up_ptr[i + 1] - c.up_ptr[i], 0, Hb);
 #pragma unroll
     for (int q = 0; q < 9; ++q) H[q] = ld(Hb[q]);
   } else {
@@ -349,7 +350,9 @@ __device__ __forceinline__ void condense_quad(const CondenseArgs<HT>& c, int64_t
   const HT* cp = c.cpl + k * 32;
   double H[3], g;
   {
-    const HT* h = kUpd == CC_UPDATE_CD ? c.bsr + (int64_t)c.up_ptr[i] * 12 + 4 * r : cp + 18 + 3 * r;
+    const HT* h = kUpd == CC_UPDATE_CD
+                      ? c.bsr + block_row_at<HT>(c.up_ptr[i], c.up_ptr[i + 1] - c.up_ptr[i], 0, r)
+                      : cp + 18 + 3 * r;
 #pragma unroll
     for (int q = 0; q < 3; ++q) H[q] = (double)h[q];
   }
@@ -588,7 +591,7 @@ __global__ void __launch_bounds__(kThreads) k_couple(
         const unsigned code = codes[off + q];
         if (code == Codes::kNone) continue;
         HT H[9];
-        load_block(bsr, (int64_t)P + q, H);
+        load_block(bsr, P, L, q, H);
         if (code == Codes::kSelf) {
           if (kUpd == CC_UPDATE_CC) mat3_tmul_acc(H, Uj, A);
         } else if (code == Codes::kDiag) {
@@ -623,7 +626,7 @@ __global__ void __launch_bounds__(kThreads) k_couple(
         const unsigned code = codes[off + q];
         if (code == Codes::kNone) continue;
         HT H[9];
-        load_block(bsr, (int64_t)P + q, H);
+        load_block(bsr, P, L, q, H);
         if (code == Codes::kDiag) {
 #pragma unroll
           for (int c = 0; c < 9; ++c) cpl[(int64_t)blockIdx.x * 32 + 18 + c] = H[c];
@@ -743,7 +746,7 @@ __global__ void __launch_bounds__(32 * kWarps) k_couple_warp(
       const unsigned code = smap[c0 + q];
       if (code == Codes::kNone) continue;
       HT H[9];
-      load_block(bsr, (int64_t)rstart[r] + (q - roff[r]), H);
+      load_block(bsr, rstart[r], rend - roff[r], q - roff[r], H);
       if (r < m) {
         const HT* Uj = Us + 9 * r;
         if (code == Codes::kSelf) {
@@ -858,13 +861,14 @@ void launch_couple_warp(Mesh& m, const int32_t* verts, int64_t count, const HT* 
 template <int kThreads, int kUpd, bool kFuse>
 __global__ void __launch_bounds__(kThreads, 1024 / kThreads) k_couple_pairs(
     const int32_t* __restrict__ verts, int64_t count, const int4* __restrict__ hdr,
-    const int32_t* __restrict__ sup_idx, const int32_t* __restrict__ sup_row, const float* __restrict__ U,
-    const uint32_t* __restrict__ list, const float* __restrict__ bsr, const float* __restrict__ g_hi, int sup_max,
-    const float* __restrict__ rot, float* __restrict__ cpl, CondenseArgs<float> ca) {
+    const int32_t* __restrict__ sup_idx, const int2* __restrict__ sup_row, const float* __restrict__ U,
+    const uint32_t* __restrict__ list, const float* __restrict__ bsr, const float* __restrict__ g_hi,
+    const float4* __restrict__ diag_g, int sup_max, const float* __restrict__ rot, float* __restrict__ cpl,
+    CondenseArgs<float> ca) {
   pdl_entry();
   extern __shared__ __align__(16) unsigned char smem[];
   float* Us = reinterpret_cast<float*>(smem);  // [m][3][4]
-  int* rstart = reinterpret_cast<int*>(smem + align16((size_t)sup_max * 12 * sizeof(float)));  // [m + 1]
+  int2* rows = reinterpret_cast<int2*>(smem + align16((size_t)sup_max * 12 * sizeof(float)));  // [m + 1] start, blocks
   constexpr int kWarps = kThreads / 32;
   __shared__ float red[kWarps][18];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -874,21 +878,30 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) k_couple_pairs(
   const uint32_t* L = list + ((int64_t)(uint32_t)hb.x | ((int64_t)hb.y << 32));
   uint32_t next = tid < np ? __ldg(L + tid) : 0u;
   stage_basis<float, 12, 4>(Us, U, rot, sup_idx, s0, m, tid, kThreads);
-  for (int s = tid; s < m; s += kThreads) rstart[s] = __ldg(sup_row + s0 + s);
-  if (tid == 0) rstart[m] = hb.z;
+  for (int s = tid; s < m; s += kThreads) rows[s] = __ldg(sup_row + s0 + s);
+  if (tid == 0) rows[m] = make_int2(hb.z, hb.w);
   float* out = cpl + (int64_t)blockIdx.x * 32;
-  if (tid < 9) out[18 + tid] = __ldg(bsr + (int64_t)hb.z * 12 + 4 * (tid / 3) + tid % 3);
+  if (tid < 9) out[18 + tid] = __ldg(bsr + block_row_at<float>(hb.z, hb.w, 0, tid / 3) + tid % 3);
   __syncthreads();
 
   float M[9], A[9], b[3] = {0, 0, 0};
   mat3_zero(M);
   mat3_zero(A);
   for (int r = tid; r < m; r += kThreads) {
-    float H[9], Uj[9], T[9];
+    float H[9], Uj[9], T[9], g0, g1, g2;
     const int j = __ldg(sup_idx + s0 + r);
-    load_block(bsr, (int64_t)rstart[r], H);
     load_slot(Us + 12 * r, Uj);
-    const float g0 = g_hi[3 * (int64_t)j], g1 = g_hi[3 * (int64_t)j + 1], g2 = g_hi[3 * (int64_t)j + 2];
+    if (diag_g) {
+      const float4 a = diag_g[3 * (int64_t)j], h = diag_g[3 * (int64_t)j + 1], c = diag_g[3 * (int64_t)j + 2];
+      H[0] = a.x; H[1] = H[3] = a.y; H[2] = H[6] = a.z; H[4] = a.w; H[5] = H[7] = h.x; H[8] = h.y;
+      g0 = h.z; g1 = h.w; g2 = c.x;
+    } else {
+      const int2 row = rows[r];
+      load_block(bsr, row.x, row.y, 0, H);
+      g0 = g_hi[3 * (int64_t)j];
+      g1 = g_hi[3 * (int64_t)j + 1];
+      g2 = g_hi[3 * (int64_t)j + 2];
+    }
     mat3_zero(T);
     mat3_mul_acc(H, Uj, T);
 #pragma unroll
@@ -902,7 +915,8 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) k_couple_pairs(
     if (e + kThreads < np) next = __ldg(L + e + kThreads);
     const int r = w & 1023, l = (w >> 10) & 1023;
     float H[9], Ul[9], Uj[9], T[9];
-    load_block(bsr, (int64_t)(rstart[r] + (int)(w >> 20)), H);
+    const int2 row = rows[r];
+    load_block(bsr, row.x, row.y, (int)(w >> 20), H);
     load_slot(Us + 12 * l, Ul);
     mat3_zero(T);
     mat3_mul_acc(H, Ul, T);
@@ -915,7 +929,8 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) k_couple_pairs(
       const int r = w & 1023, l = (w >> 10) & 1023;
       const bool lower = l == (int)kPairSelf;  // stored as H_ji, j = row r of the support
       float H[9], Uv[9];
-      load_block(bsr, (int64_t)(rstart[r] + (int)(w >> 20)), H);
+      const int2 row = rows[r];
+      load_block(bsr, row.x, row.y, (int)(w >> 20), H);
       load_slot(Us + 12 * (lower ? r : l), Uv);
       if (lower) {
         float t;
@@ -972,15 +987,15 @@ void launch_couple_pairs(Mesh& m, const int32_t* verts, int64_t count, const flo
                          const float* g_hi, float* cpl, const float* rot, const CondenseArgs<float>& ca, bool fuse,
                          cudaStream_t s) {
   const int supm = m.sup_max > 0 ? m.sup_max : 1;
-  const size_t smem = align16((size_t)supm * 12 * sizeof(float)) + align16((size_t)(supm + 1) * 4);
+  const size_t smem = align16((size_t)supm * 12 * sizeof(float)) + (size_t)(supm + 1) * sizeof(int2);
   // the limit on supports is the one of the slot-map kernels, whichever kernel runs
   CCG_CHECK(kThreads == 32 || cta_smem_bytes<float>(supm, m.smap_max, m.smap_wide ? 2 : 1, kThreads) <= 220 * 1024,
             CC_ERR_INVALID_ARG, "support too large for the coupling kernel");
   auto go = [&](auto kern) {
     set_smem_limit(reinterpret_cast<const void*>(kern), smem);
     pdl_launch(kern, (unsigned)count, kThreads, smem, s, verts, count, (const int4*)m.d_pair_hdr.p,
-               (const int32_t*)m.d_sup_idx.p, (const int32_t*)m.d_sup_row.p, U, (const uint32_t*)m.d_pairs.p, bsr,
-               g_hi, supm, rot, cpl, ca);
+               (const int32_t*)m.d_sup_idx.p, (const int2*)m.d_sup_row.p, U, (const uint32_t*)m.d_pairs.p, bsr,
+               g_hi, rows_from_positions(m, true) ? (const float4*)m.mx.diag_g.p : nullptr, supm, rot, cpl, ca);
   };
   if (fuse) go(k_couple_pairs<kThreads, kUpd, true>);
   else go(k_couple_pairs<kThreads, kUpd, false>);
