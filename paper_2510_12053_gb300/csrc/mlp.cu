@@ -313,25 +313,33 @@ __global__ void k_basis_residual(int nrows, const int32_t* __restrict__ rows, co
 // A training minibatch's inputs: dst row b = src row idx[*step * B + b], and
 // dstt = dst^T, in 32 x 32 tiles through shared memory (the step counter lives
 // on the device, so one captured step replays for all).  Columns past `cols`
-// up to ldd are copied too (the GEMM's padded width).
+// up to ldd are copied too (the GEMM's padded width).  32 x 8 threads.
 __global__ void k_gather_inputs(const bf16* __restrict__ src, int64_t lds, const int32_t* __restrict__ idx,
                                 const int* __restrict__ step, int B, int cols, bf16* __restrict__ dst, int64_t ldd,
                                 bf16* __restrict__ dstt, int64_t lddt) {
   __shared__ bf16 tile[32][33];
   const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32, c = c0 + threadIdx.x;
   const int32_t* rows = idx + (int64_t)*step * B;
-  for (int k = threadIdx.y; k < 32; k += blockDim.y) {
-    const int r = r0 + k;
+  int row[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int r = r0 + threadIdx.y + 8 * q;
+    row[q] = r < B ? rows[r] : 0;
+  }
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int k = threadIdx.y + 8 * q, r = r0 + k;
     if (r < B && c < ldd) {
-      const bf16 v = src[(int64_t)rows[r] * lds + c];
+      const bf16 v = src[(int64_t)row[q] * lds + c];
       dst[(int64_t)r * ldd + c] = v;
       tile[k][threadIdx.x] = v;
     }
   }
   __syncthreads();
-  for (int k = threadIdx.y; k < 32; k += blockDim.y) {
-    const int ct = c0 + k, r = r0 + threadIdx.x;
-    if (r < B && ct < cols) dstt[(int64_t)ct * lddt + r] = tile[threadIdx.x][k];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int ct = c0 + threadIdx.y + 8 * q, r = r0 + threadIdx.x;
+    if (r < B && ct < cols) dstt[(int64_t)ct * lddt + r] = tile[threadIdx.x][threadIdx.y + 8 * q];
   }
 }
 
@@ -363,11 +371,25 @@ __global__ void k_loss_dy(const float* __restrict__ Y, int64_t ldy, const float*
   __shared__ double red[8];
   const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
   const int32_t* rows = idx ? idx + (int64_t)*step * B : nullptr;
+  // all of a thread's loads are issued before the first is used
+  const int c = c0 + threadIdx.x;
+  int row[4];
+  float y[4], t[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int r = r0 + threadIdx.y + 8 * q;
+    row[q] = r < B && rows ? rows[r] : r;
+    if (r < B && c < D) y[q] = Y[(int64_t)r * ldy + c];
+  }
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+    if (r0 + (int)threadIdx.y + 8 * q < B && c < D) t[q] = T[(int64_t)row[q] * ldt + c];
   float acc = 0.0f;  // a thread's four squares in float32; the block's warps' sums in float64
-  for (int k = threadIdx.y; k < 32; k += blockDim.y) {
-    const int r = r0 + k, c = c0 + threadIdx.x;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int k = threadIdx.y + 8 * q, r = r0 + k;
     if (r < B && c < D) {
-      const float d = Y[(int64_t)r * ldy + c] - T[(int64_t)(rows ? rows[r] : r) * ldt + c];
+      const float d = y[q] - t[q];
       acc = fmaf(d, d, acc);
       const bf16 g = __float2bfloat16_rn(d * scale);
       dy[(int64_t)r * lddy + c] = g;
@@ -378,9 +400,10 @@ __global__ void k_loss_dy(const float* __restrict__ Y, int64_t ldy, const float*
   for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
   if (threadIdx.x == 0) red[threadIdx.y] = (double)acc;
   __syncthreads();
-  for (int k = threadIdx.y; k < 32; k += blockDim.y) {
-    const int c = c0 + k, r = r0 + threadIdx.x;
-    if (r < B && c < D) dyt[(int64_t)c * lddt + r] = tile[threadIdx.x][k];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int ct = c0 + threadIdx.y + 8 * q, r = r0 + threadIdx.x;
+    if (r < B && ct < D) dyt[(int64_t)ct * lddt + r] = tile[threadIdx.x][threadIdx.y + 8 * q];
   }
   if (threadIdx.x == 0 && threadIdx.y == 0) {
     double sum = 0.0;
@@ -429,6 +452,7 @@ __device__ __forceinline__ float row_sum_bf16(const bf16* __restrict__ src, int6
   float a = 0.0f;
   if ((lds & 1) == 0 && (cols & 1) == 0 && (reinterpret_cast<uintptr_t>(src) & 3) == 0) {
     const __nv_bfloat162* row2 = reinterpret_cast<const __nv_bfloat162*>(row);
+#pragma unroll 8
     for (int c = threadIdx.x; c < cols / 2; c += 256) {
       const float2 f = __bfloat1622float2(row2[c]);
       a += f.x + f.y;
@@ -491,8 +515,9 @@ __global__ void k_adam(AdamArgs a, const float* __restrict__ g, int64_t count, f
 // gradient from what the backward pass left behind, Adam, and the BF16 copies.
 // Blocks [wblk[l], wblk[l + 1]) take 32 x 32 tiles of W_l, whose split-K slices
 // they sum (ascending); the blocks after them one bias each, the sum of a row
-// of dZ_l^T.  As four launches a layer and six more, at 4-6 us each, this took
-// 62 us of a 236 us step (network 258-3x256-576, batch 8 192).
+// of dZ_l^T.  Bound by the latency of the slices' loads (L2), hence eight at a
+// time.  Network 258-3x256-576, batch 8 192: 19 us cold, where the separate
+// sums, row sums, Adam and conversions were thirteen launches of 4-6 us.
 constexpr int kUpdMaxLayers = 8;  // layers of one launch (deeper networks take several)
 struct UpdateArgs {
   int L, B;
@@ -522,36 +547,65 @@ __global__ void __launch_bounds__(256) k_train_update(const __grid_constant__ Up
   while (blk >= u.wblk[l + 1]) ++l;
   const int N = u.N[l], K = u.K[l], S = u.S[l], t = blk - u.wblk[l];
   const int n0 = (t / u.tiles_k[l]) * 32, k0 = (t % u.tiles_k[l]) * 32;
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   const int64_t stride = (int64_t)N * K;
-  const float* P = u.slices[l];
   __shared__ bf16 tile[32][33];
-  float g[4] = {0.f, 0.f, 0.f, 0.f};
-  const int k = k0 + tx;
-  if (k < K) {
-#pragma unroll 8
-    for (int s = 0; s < S; ++s) {
+  {  // four neighbouring weights a thread
+    const int nl = threadIdx.x >> 3, kl = (threadIdx.x & 7) * 4, n = n0 + nl, k = k0 + kl;
+    const float* P = u.slices[l] + (int64_t)n * K + k;
+    float g[4] = {0.f, 0.f, 0.f, 0.f};
+    if (n < N && (K & 3) == 0 && k < K) {
+      int s = 0;
+      for (; s + 8 <= S; s += 8) {  // eight loads in flight, summed in order
+        float4 v[8];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int n = n0 + ty + 8 * q;
-        if (n < N) g[q] += P[s * stride + (int64_t)n * K + k];
+        for (int i = 0; i < 8; ++i) v[i] = __ldcg(reinterpret_cast<const float4*>(P + (s + i) * stride));
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          g[0] += v[i].x;
+          g[1] += v[i].y;
+          g[2] += v[i].z;
+          g[3] += v[i].w;
+        }
       }
-    }
-  }
+      for (; s < S; ++s) {
+        const float4 v = __ldcg(reinterpret_cast<const float4*>(P + s * stride));
+        g[0] += v.x;
+        g[1] += v.y;
+        g[2] += v.z;
+        g[3] += v.w;
+      }
+    } else if (n < N) {
+      int s = 0;
+      for (; s + 4 <= S; s += 4) {
+        float v[4][4];
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int n = n0 + ty + 8 * q;
-    if (n < N && k < K) {
-      const bf16 w = __float2bfloat16_rn(adam_update(a, u.off_w[l] + (int64_t)n * K + k, g[q], bc1, bc2));
-      u.w16[l][(int64_t)n * u.ldk[l] + k] = w;
-      tile[ty + 8 * q][tx] = w;
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) v[i][q] = k + q < K ? __ldcg(P + (s + i) * stride + q) : 0.0f;
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) g[q] += v[i][q];
+      }
+      for (; s < S; ++s)
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (k + q < K) g[q] += __ldcg(P + s * stride + q);
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if (n < N && k + q < K) {
+        const bf16 w = __float2bfloat16_rn(adam_update(a, u.off_w[l] + (int64_t)n * K + k + q, g[q], bc1, bc2));
+        u.w16[l][(int64_t)n * u.ldk[l] + k + q] = w;
+        tile[nl][kl + q] = w;
+      }
     }
   }
   __syncthreads();
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
-    const int kk = k0 + ty + 8 * q, n = n0 + tx;
-    if (n < N && kk < K) u.wt16[l][(int64_t)kk * u.ldn[l] + n] = tile[tx][ty + 8 * q];
+    const int tx = threadIdx.x & 31, kk = (threadIdx.x >> 5) + 8 * q, n = n0 + tx;
+    if (n < N && k0 + kk < K) u.wt16[l][(int64_t)(k0 + kk) * u.ldn[l] + n] = tile[tx][kk];
   }
 }
 

@@ -1179,24 +1179,38 @@ void mlp_forward_fused(const void* X, int64_t ldx, int M, const std::vector<int>
 }
 
 GemmShape gemm_pick_shape(int M, int N, int K, bool allow_split) {
-  // the persistent kernel keeps one CTA per SM; aim for at least one tile per SM
+  // The persistent kernel keeps one CTA per SM.  A candidate's cost is what the
+  // busiest CTA does: its tiles, each bn columns and about 32 more for the
+  // tile's own start and end; equal costs go to the wider tile, which reads A
+  // less often.  (The widest tile that filled every SM, which this replaces,
+  // gave the 8 192 x 576 output layer 192-column tiles, two on 40 SMs and one on
+  // the rest, and the 256 x 256 weight gradients 64 CTAs.)
   const int slots = num_sms();
   GemmShape sh;
-  const int mt = (M + kBM - 1) / kBM;
+  const int mt = (M + kBM - 1) / kBM, kt = (K + kBK - 1) / kBK;
   const int cands[4] = {256, 192, 128, 64};
-  sh.bn = 64;
+  auto tiles_of = [&](int bn) { return (int64_t)mt * ((N + bn - 1) / bn); };
+  if (allow_split) {
+    // slices for one CTA per SM with the widest tile, of at least four K steps
+    // each: a function of K that never falls, which a workspace can be sized by
+    int wide = 64;
+    for (int bn : cands)
+      if (N % bn == 0) {
+        wide = bn;
+        break;
+      }
+    const int64_t want = (slots + tiles_of(wide) - 1) / tiles_of(wide);
+    sh.splits = (int)std::max<int64_t>(1, std::min<int64_t>(want, kt / 4));
+  }
+  const int per = (kt + sh.splits - 1) / sh.splits, slices = (kt + per - 1) / per;
+  int64_t best = -1;
   for (int bn : cands) {
     if (N % bn != 0 && bn != 64) continue;
-    if ((int64_t)mt * ((N + bn - 1) / bn) >= slots || allow_split) {
+    const int64_t rounds = (tiles_of(bn) * slices + slots - 1) / slots, cost = rounds * (bn + 32);
+    if (best < 0 || cost < best) {
+      best = cost;
       sh.bn = bn;
-      break;
     }
-  }
-  if (allow_split) {
-    const int tiles = mt * ((N + sh.bn - 1) / sh.bn);
-    const int kt = (K + kBK - 1) / kBK;
-    const int want = (slots + tiles - 1) / tiles;
-    sh.splits = std::max(1, std::min(want, kt / 4));
   }
   return sh;
 }
