@@ -848,6 +848,48 @@ void launch_couple_warp(Mesh& m, const int32_t* verts, int64_t count, const HT* 
   CCG_CUDA(cudaGetLastError());
 }
 
+// The coupling CTA's 18 sums (Ht = M + M^T, A, b) in a fixed order, to out[0..17]:
+// sixteen values halved over the lanes (lane L ends with value (L >> 1) reversed
+// in four bits), the last two by a butterfly each, then the warps' sums in order.
+template <typename HT, int kWarps>
+__device__ __forceinline__ void reduce18(const HT* M, const HT* A, const HT* b, HT (*red)[18], HT* __restrict__ out) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  HT v[16] = {2 * M[0], M[1] + M[3], M[2] + M[6], 2 * M[4], M[5] + M[7], 2 * M[8],
+                 A[0], A[1], A[2], A[3], A[4], A[5], A[6], A[7], A[8], b[0]};
+#pragma unroll
+  for (int o = 16, h = 8; h > 0; o >>= 1, h >>= 1) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int q = 0; q < h; ++q) {
+      const HT keep = up ? v[q + h] : v[q], send = up ? v[q] : v[q + h];
+      v[q] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+  v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+  const HT b1 = warp_sum(b[1]), b2 = warp_sum(b[2]);
+  const int mine = ((lane & 16) >> 1) | ((lane & 8) >> 1) | ((lane & 4) >> 1) | ((lane & 2) >> 1);
+  if constexpr (kWarps == 1) {
+    if ((lane & 1) == 0) out[mine] = v[0];
+    if (lane == 0) {
+      out[16] = b1;
+      out[17] = b2;
+    }
+  } else {
+    if ((lane & 1) == 0) red[warp][mine] = v[0];
+    if (lane == 0) {
+      red[warp][16] = b1;
+      red[warp][17] = b2;
+    }
+    __syncthreads();
+    if (tid < 18) {
+      HT t = red[0][tid];
+#pragma unroll
+      for (int q = 1; q < kWarps; ++q) t += red[q][tid];
+      out[tid] = t;
+    }
+  }
+}
+
 // Float32 coupling products, one CTA per free vertex i of the list, from the
 // vertex's pair list (Mesh::d_pairs).  Three loops without divergence:
 //   support rows j      1/2 H_jj's share of Ht and U_j^T g_j, a row per thread;
@@ -942,43 +984,7 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) k_couple_pairs(
     }
   }
 
-  // the CTA's sums in a fixed order: sixteen values halved over the lanes
-  // (lane L ends with value (L >> 1) reversed in four bits), the last two by a
-  // butterfly each, then the warps' sums in order
-  float v[16] = {2.f * M[0], M[1] + M[3], M[2] + M[6], 2.f * M[4], M[5] + M[7], 2.f * M[8],
-                 A[0], A[1], A[2], A[3], A[4], A[5], A[6], A[7], A[8], b[0]};
-#pragma unroll
-  for (int o = 16, h = 8; h > 0; o >>= 1, h >>= 1) {
-    const bool up = (lane & o) != 0;
-#pragma unroll
-    for (int q = 0; q < h; ++q) {
-      const float keep = up ? v[q + h] : v[q], send = up ? v[q] : v[q + h];
-      v[q] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-    }
-  }
-  v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
-  const float b1 = warp_sum(b[1]), b2 = warp_sum(b[2]);
-  const int mine = ((lane & 16) >> 1) | ((lane & 8) >> 1) | ((lane & 4) >> 1) | ((lane & 2) >> 1);
-  if constexpr (kWarps == 1) {
-    if ((lane & 1) == 0) out[mine] = v[0];
-    if (lane == 0) {
-      out[16] = b1;
-      out[17] = b2;
-    }
-  } else {
-    if ((lane & 1) == 0) red[warp][mine] = v[0];
-    if (lane == 0) {
-      red[warp][16] = b1;
-      red[warp][17] = b2;
-    }
-    __syncthreads();
-    if (tid < 18) {
-      float t = red[0][tid];
-#pragma unroll
-      for (int q = 1; q < kWarps; ++q) t += red[q][tid];
-      out[tid] = t;
-    }
-  }
+  reduce18<float, kWarps>(M, A, b, red, out);
   if constexpr (kFuse) condense_group_tail<double, float, true, kUpd>(ca, 1e-12);
 }
 
@@ -999,6 +1005,136 @@ void launch_couple_pairs(Mesh& m, const int32_t* verts, int64_t count, const flo
   };
   if (fuse) go(k_couple_pairs<kThreads, kUpd, true>);
   else go(k_couple_pairs<kThreads, kUpd, false>);
+  CCG_CUDA(cudaGetLastError());
+}
+
+// Float64 coupling products, one CTA per free vertex i, from its pair list.
+// The float64 pipe bounds it: a warp instruction takes one of its sub-partitions
+// about 61 cycles however many lanes work, so what counts is float64 instructions
+// per warp.  A thread takes a support row j and sums Z_j = 1/2 H_jj U_j +
+// sum_l H_jl U_l over the row's pairs (27 instructions each), folding it with
+// U_j once; rows are dealt out by falling length, so the lanes of a warp have
+// rows of about one length.  An interior 2-ring (64 rows of 0 to 7 pairs) takes
+// about 520 warp instructions, where four threads a row, with diagonal blocks
+// and blocks with i in branches of their own, took 1 460 (251 us a colour of
+// 3 450 vertices).  A float64 sweep of the 24 x 23 x 25 box: 1.34 -> 0.82 ms.
+template <int kThreads, int kUpd, bool kFuse>
+__global__ void __launch_bounds__(kThreads, 512 / kThreads) k_couple_rows64(
+    const int32_t* __restrict__ verts, int64_t count, const int4* __restrict__ hdr,
+    const int32_t* __restrict__ sup_idx, const int2* __restrict__ sup_row, const double* __restrict__ U,
+    const uint32_t* __restrict__ list, const double* __restrict__ bsr, const double* __restrict__ g, int sup_max,
+    const double* __restrict__ rot, double* __restrict__ cpl, CondenseArgs<double> ca) {
+  pdl_entry();
+  extern __shared__ __align__(16) unsigned char smem[];
+  double* Us = reinterpret_cast<double*>(smem);                                                    // [m][3][4]
+  int2* rows = reinterpret_cast<int2*>(smem + align16((size_t)sup_max * 12 * sizeof(double)));     // [m + 1] start, blocks
+  int2* span = rows + (sup_max + 1);                                                               // [m] the row's pairs
+  int* order = reinterpret_cast<int*>(span + sup_max);                                             // [m] rows, longest first
+  constexpr int kWarps = kThreads / 32;
+  __shared__ double red[kWarps][18];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int i = verts[blockIdx.x];
+  const int4 ha = __ldg(hdr + 2 * (int64_t)i), hb = __ldg(hdr + 2 * (int64_t)i + 1);
+  const int s0 = ha.x, m = ha.y, np = ha.z, ns = ha.w;
+  const uint32_t* L = list + ((int64_t)(uint32_t)hb.x | ((int64_t)hb.y << 32));
+  stage_basis<double, 12, 4>(Us, U, rot, sup_idx, s0, m, tid, kThreads);
+  for (int s = tid; s < m; s += kThreads) {
+    rows[s] = __ldg(sup_row + s0 + s);
+    span[s] = make_int2(0, 0);
+  }
+  if (tid == 0) rows[m] = make_int2(hb.z, hb.w);
+  double* out = cpl + (int64_t)blockIdx.x * 32;
+  if (tid < 9) out[18 + tid] = __ldg(bsr + block_row_at<double>(hb.z, hb.w, 0, tid / 3) + tid % 3);
+  __syncthreads();
+  for (int e = tid; e < np; e += kThreads) {  // the list is in row order
+    const int r = __ldg(L + e) & 1023;
+    if (e == 0 || (int)(__ldg(L + e - 1) & 1023) != r) span[r].x = e;
+    if (e == np - 1 || (int)(__ldg(L + e + 1) & 1023) != r) span[r].y = e + 1;
+  }
+  __syncthreads();
+  for (int s = tid; s < m; s += kThreads) {
+    const int len = span[s].y - span[s].x;
+    int rank = 0;
+    for (int q = 0; q < m; ++q) {
+      const int other = span[q].y - span[q].x;
+      rank += other > len || (other == len && q < s);
+    }
+    order[rank] = s;
+  }
+  __syncthreads();
+
+  double M[9], A[9], b[3] = {0, 0, 0};
+  mat3_zero(M);
+  mat3_zero(A);
+  for (int k = tid; k < m; k += kThreads) {
+    const int r = order[k];
+    const int2 row = rows[r], sp = span[r];
+    double H[9], Z[9];
+    mat3_zero(Z);
+    {
+      double Uj[9];
+      load_block(bsr, row.x, row.y, 0, H);
+      load_slot(Us + 12 * r, Uj);
+      mat3_mul_acc(H, Uj, Z);
+#pragma unroll
+      for (int c = 0; c < 9; ++c) Z[c] *= 0.5;
+    }
+    for (int e = sp.x; e < sp.y; ++e) {
+      const uint32_t w = __ldg(L + e);
+      double Ul[9];
+      load_block(bsr, row.x, row.y, (int)(w >> 20), H);
+      load_slot(Us + 12 * (int)((w >> 10) & 1023), Ul);
+      mat3_mul_acc(H, Ul, Z);
+    }
+    double Uj[9];
+    load_slot(Us + 12 * r, Uj);
+    mat3_tmul_acc(Uj, Z, M);
+    const int j = __ldg(sup_idx + s0 + r);
+    const double g0 = g[3 * (int64_t)j], g1 = g[3 * (int64_t)j + 1], g2 = g[3 * (int64_t)j + 2];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) b[c] = fma(Uj[6 + c], g2, fma(Uj[3 + c], g1, fma(Uj[c], g0, b[c])));
+  }
+  if (kUpd == CC_UPDATE_CC) {
+    for (int e = tid ^ (kThreads / 2); e < ns; e += kThreads) {  // the second half's rows are the short ones
+      const uint32_t w = __ldg(L + np + e);
+      const int r = w & 1023, l = (w >> 10) & 1023;
+      const bool lower = l == (int)kPairSelf;  // stored as H_ji, j = row r of the support
+      double H[9], Uv[9];
+      const int2 row = rows[r];
+      load_block(bsr, row.x, row.y, (int)(w >> 20), H);
+      load_slot(Us + 12 * (lower ? r : l), Uv);
+      if (lower) {
+        double t;
+        t = H[1]; H[1] = H[3]; H[3] = t;
+        t = H[2]; H[2] = H[6]; H[6] = t;
+        t = H[5]; H[5] = H[7]; H[7] = t;
+      }
+      mat3_mul_acc(H, Uv, A);
+    }
+  }
+  reduce18<double, kWarps>(M, A, b, red, out);
+  if constexpr (kFuse) condense_group_tail<double, double, false, kUpd>(ca, 1e-12);
+}
+
+template <int kThreads, int kUpd>
+void launch_couple_rows64(Mesh& m, const int32_t* verts, int64_t count, const double* U, const double* bsr,
+                          const double* g, double* cpl, const double* rot, const CondenseArgs<double>& ca, bool fuse,
+                          cudaStream_t s) {
+  const int supm = m.sup_max > 0 ? m.sup_max : 1;
+  const size_t smem = align16((size_t)supm * 12 * sizeof(double)) + (size_t)(supm + 1) * sizeof(int2) +
+                      (size_t)supm * (sizeof(int2) + sizeof(int));
+  // the limit on supports is the one of the slot-map kernels, whichever kernel runs
+  const size_t limit = kThreads == 32 ? warp_smem_bytes<double>(supm, 4)
+                                      : cta_smem_bytes<double>(supm, m.smap_max, m.smap_wide ? 2 : 1, kThreads);
+  CCG_CHECK(limit <= 220 * 1024, CC_ERR_INVALID_ARG, "support too large for the coupling kernel");
+  auto go = [&](auto kern) {
+    set_smem_limit(reinterpret_cast<const void*>(kern), smem);
+    pdl_launch(kern, (unsigned)count, kThreads, smem, s, verts, count, (const int4*)m.d_pair_hdr.p,
+               (const int32_t*)m.d_sup_idx.p, (const int2*)m.d_sup_row.p, U, (const uint32_t*)m.d_pairs.p, bsr, g, supm,
+               rot, cpl, ca);
+  };
+  if (fuse) go(k_couple_rows64<kThreads, kUpd, true>);
+  else go(k_couple_rows64<kThreads, kUpd, false>);
   CCG_CUDA(cudaGetLastError());
 }
 
@@ -1030,6 +1166,14 @@ void launch_one(Mesh& m, const int32_t* verts, int64_t count, const HT* U, const
           case 256: launch_couple_pairs<256, kUpd>(m, verts, count, U, bsr, g_hi, cpl, rot, cf, fuse, s); break;
           default: launch_couple_pairs<128, kUpd>(m, verts, count, U, bsr, g_hi, cpl, rot, cf, fuse, s);
         }
+      }
+    } else if (m.pairs_ok) {
+      done = true;
+      switch (m.tune_couple_threads) {
+        case 32: launch_couple_rows64<32, kUpd>(m, verts, count, U, bsr, g64, cpl, rot, cf, fuse, s); break;
+        case 64: launch_couple_rows64<64, kUpd>(m, verts, count, U, bsr, g64, cpl, rot, cf, fuse, s); break;
+        case 256: launch_couple_rows64<256, kUpd>(m, verts, count, U, bsr, g64, cpl, rot, cf, fuse, s); break;
+        default: launch_couple_rows64<128, kUpd>(m, verts, count, U, bsr, g64, cpl, rot, cf, fuse, s);
       }
     }
     if (!done) switch (m.tune_couple_threads) {
