@@ -192,7 +192,7 @@ __device__ __forceinline__ void tet_grad_f64_body(const int4* __restrict__ tets,
   if (fcr) {
     // lh holds lam for this material
     const double nan = __longlong_as_double(0x7ff8000000000000ll);
-    if (!polar_newton<double>(kin.F, R))
+    if (!polar_f64(kin.F, R))
       for (int q = 0; q < 9; ++q) R[q] = nan;
     const double sl = lh * (kin.J - 1.0);
 #pragma unroll
@@ -557,7 +557,7 @@ __global__ void k_energy_tets(const int4* __restrict__ tets, const double* __res
     if (kFCR) {
       double R[9];
       double d2 = 0.0;
-      if (polar_newton<double>(kin.F, R)) {
+      if (polar_f64(kin.F, R)) {
 #pragma unroll
         for (int q = 0; q < 9; ++q) d2 += (kin.F[q] - R[q]) * (kin.F[q] - R[q]);
       } else {
@@ -604,7 +604,7 @@ __global__ void k_energy_mesh(const int64_t* __restrict__ tptr, const int64_t* _
     if (kFCR) {
       double R[9];
       double d2 = 0.0;
-      if (polar_newton<double>(kin.F, R)) {
+      if (polar_f64(kin.F, R)) {
 #pragma unroll
         for (int q = 0; q < 9; ++q) d2 += (kin.F[q] - R[q]) * (kin.F[q] - R[q]);
       } else {
