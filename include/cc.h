@@ -446,8 +446,10 @@ cc_status cc_autotune(cc_mesh* mesh, const double* x_dev, const double* xtilde_d
 /* Sets the launch shapes cc_autotune chooses among (no counterpart in the
  * paper): couple_threads in {32 (one warp per vertex), 64, 128, 256},
  * gather_warps in {2, 4, 8}, couple_row_lanes (threads sharing one block row
- * of the support in the coupling kernel with 64 or more threads) in
- * {1, 2, 4, 8}; 0 keeps the current value.  CC_ERR_INVALID_ARG for any other
+ * of the support in the slot-map coupling kernel with 64 or more threads, which
+ * the mixed path of dynamic meshes and supports of more than 1 020 vertices run;
+ * the others take a block or a row per thread) in {1, 2, 4, 8}; 0 keeps the
+ * current value.  CC_ERR_INVALID_ARG for any other
  * value. */
 cc_status cc_set_launch_shape(cc_mesh* mesh, int32_t couple_threads, int32_t gather_warps, int32_t couple_row_lanes);
 

@@ -493,6 +493,8 @@ __device__ __forceinline__ void condense_group_tail(const CondenseArgs<HT>& c, A
   if (k < c.count) condense_vertex<AR, HT, kMixed, kUpd>(c, k, rel);
 }
 
+// The slot-map kernel, for the float32 path of dynamic meshes (whose sums it
+// keeps in their order) and supports that the pair lists' fields do not hold.
 // Coupling products, one CTA per free vertex i of the list.  Groups of
 // 2^row_lanes_log2 threads take the block rows of the support S and of i
 // itself; a group's threads take the row's upper blocks (H_jl, l >= j)
@@ -506,7 +508,7 @@ __device__ __forceinline__ void condense_group_tail(const CondenseArgs<HT>& c, A
 // b (3), H_ii (9, stored directly by the thread that reads it).
 // kFuse: the CTA then takes part in the group condensation (condense_group_tail).
 template <typename HT, typename SlotT, bool kMixed, int kUpd, int kThreads, bool kFuse = false>
-__global__ void __launch_bounds__(kThreads) k_couple(
+__global__ void __launch_bounds__(kThreads, sizeof(HT) == 4 ? 1024 / kThreads : 1) k_couple(
     const int32_t* __restrict__ verts, int64_t count, const int32_t* __restrict__ sup_ptr,
     const int32_t* __restrict__ sup_idx, const HT* __restrict__ U, const int32_t* __restrict__ up_ptr,
     const int64_t* __restrict__ smap_ptr, const SlotT* __restrict__ smap, const HT* __restrict__ bsr,
@@ -594,14 +596,13 @@ __global__ void __launch_bounds__(kThreads) k_couple(
         load_block(bsr, P, L, q, H);
         if (code == Codes::kSelf) {
           if (kUpd == CC_UPDATE_CC) mat3_tmul_acc(H, Uj, A);
-        } else if (code == Codes::kDiag) {
-#pragma unroll
-          for (int c = 0; c < 9; ++c) H[c] *= HT(0.5);
-          mat3_mul_acc(H, Uj, Z);
-          any = true;
-        } else {
+        } else {  // a diagonal block is half a pair (j, j); one path, as a row's lanes hold both kinds
+          const bool dg = code == Codes::kDiag;
+          const HT w = dg ? HT(0.5) : HT(1);
           HT Ul[9];
-          load_slot(Us + 12 * (int)code, Ul);
+          load_slot(Us + 12 * (dg ? r : (int)code), Ul);
+#pragma unroll
+          for (int c = 0; c < 9; ++c) H[c] *= w;
           mat3_mul_acc(H, Ul, Z);
           any = true;
         }
@@ -900,6 +901,9 @@ __device__ __forceinline__ void reduce18(const HT* M, const HT* A, const HT* b, 
 // and Ht = M + M^T.  Every entry says which block and which basis slots it
 // needs, so a thread's list entry, block row and basis rows are all known two
 // loads after the vertex number, and no thread walks blocks outside the support.
+// Bound by L1 wavefronts (72% of peak) and load latency together: 39 us a colour
+// of the 32^3 cube (8 440 vertices) cold, 50 k wavefronts an SM; the slot-map
+// kernel above took 46 us.  64 registers (16 CTAs of 64 threads an SM).
 template <int kThreads, int kUpd, bool kFuse>
 __global__ void __launch_bounds__(kThreads, 1024 / kThreads) k_couple_pairs(
     const int32_t* __restrict__ verts, int64_t count, const int4* __restrict__ hdr,
