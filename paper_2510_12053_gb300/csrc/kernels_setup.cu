@@ -405,9 +405,20 @@ static void build_pair_lists(Mesh& m) {
                              (int)(m.up_ptr[v + 1] - m.up_ptr[v]));
     at += c.x + c.y;
   }
-  m.d_pair_hdr.upload(hdr, s);
-  m.d_sup_row.alloc(total);
-  m.d_pairs.alloc(at);
+  try {
+    m.d_pair_hdr.upload(hdr, s);
+    m.d_sup_row.alloc(total);
+    m.d_pairs.alloc(at);
+  } catch (const Fail& f) {  // no room for them: the slot-map kernels need only what follows
+    if (f.st != CC_ERR_OOM) throw;
+    cudaGetLastError();
+    clear_error();
+    m.d_pair_hdr.release();
+    m.d_sup_row.release();
+    m.d_pairs.release();
+    CCG_CUDA(cudaStreamSynchronize(s));
+    return;
+  }
   k_pair_lists<true><<<grid, 256, 0, s>>>(m.d_free_rows.p, nf, m.d_sup_ptr.p, m.d_sup_idx.p, m.d_up_ptr.p,
                                           m.d_up_col.p, nullptr, m.d_pair_hdr.p, m.d_sup_row.p, m.d_pairs.p);
   CCG_CUDA(cudaGetLastError());
