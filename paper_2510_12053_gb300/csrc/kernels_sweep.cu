@@ -852,8 +852,11 @@ void launch_couple_warp(Mesh& m, const int32_t* verts, int64_t count, const HT* 
 // The coupling CTA's 18 sums (Ht = M + M^T, A, b) in a fixed order, to out[0..17]:
 // sixteen values halved over the lanes (lane L ends with value (L >> 1) reversed
 // in four bits), the last two by a butterfly each, then the warps' sums in order.
-template <typename HT, int kWarps>
-__device__ __forceinline__ void reduce18(const HT* M, const HT* A, const HT* b, HT (*red)[18], HT* __restrict__ out) {
+// kTwo (one warp): the sums of the first of two shares wait in `sum` for the
+// second's, added as two warps' are.
+template <typename HT, int kWarps, bool kTwo = false>
+__device__ __forceinline__ void reduce18(const HT* M, const HT* A, const HT* b, HT (*red)[18], HT* __restrict__ out,
+                                         HT* sum = nullptr, int share = 0) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   HT v[16] = {2 * M[0], M[1] + M[3], M[2] + M[6], 2 * M[4], M[5] + M[7], 2 * M[8],
                  A[0], A[1], A[2], A[3], A[4], A[5], A[6], A[7], A[8], b[0]};
@@ -869,11 +872,19 @@ __device__ __forceinline__ void reduce18(const HT* M, const HT* A, const HT* b, 
   v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
   const HT b1 = warp_sum(b[1]), b2 = warp_sum(b[2]);
   const int mine = ((lane & 16) >> 1) | ((lane & 8) >> 1) | ((lane & 4) >> 1) | ((lane & 2) >> 1);
+  if constexpr (kTwo) {
+    if (share == 0) {
+      sum[0] = v[0];
+      sum[1] = b1;
+      sum[2] = b2;
+      return;
+    }
+  }
   if constexpr (kWarps == 1) {
-    if ((lane & 1) == 0) out[mine] = v[0];
+    if ((lane & 1) == 0) out[mine] = kTwo ? sum[0] + v[0] : v[0];
     if (lane == 0) {
-      out[16] = b1;
-      out[17] = b2;
+      out[16] = kTwo ? sum[1] + b1 : b1;
+      out[17] = kTwo ? sum[2] + b2 : b2;
     }
   } else {
     if ((lane & 1) == 0) red[warp][mine] = v[0];
@@ -904,7 +915,10 @@ __device__ __forceinline__ void reduce18(const HT* M, const HT* A, const HT* b, 
 // Bound by L1 wavefronts (72% of peak) and load latency together: 39 us a colour
 // of the 32^3 cube (8 440 vertices) cold, 50 k wavefronts an SM; the slot-map
 // kernel above took 46 us.  64 registers (16 CTAs of 64 threads an SM).
-template <int kThreads, int kUpd, bool kFuse>
+// kShares: the loops' work is dealt to kShares x kThreads threads, and the CTA
+// takes the shares one after the other; each share's sums are reduced by
+// themselves, so one warp with two shares gives the bits of two warps.
+template <int kThreads, int kUpd, bool kFuse, int kShares = 1>
 __global__ void __launch_bounds__(kThreads, 1024 / kThreads) k_couple_pairs(
     const int32_t* __restrict__ verts, int64_t count, const int4* __restrict__ hdr,
     const int32_t* __restrict__ sup_idx, const int2* __restrict__ sup_row, const float* __restrict__ U,
@@ -916,13 +930,14 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) k_couple_pairs(
   float* Us = reinterpret_cast<float*>(smem);  // [m][3][4]
   int2* rows = reinterpret_cast<int2*>(smem + align16((size_t)sup_max * 12 * sizeof(float)));  // [m + 1] start, blocks
   constexpr int kWarps = kThreads / 32;
+  constexpr int kStep = kThreads * kShares;  // threads the work is dealt to
+  static_assert(kShares == 1 || kWarps == 1, "shares are summed by one warp");
   __shared__ float red[kWarps][18];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int i = verts[blockIdx.x];
   const int4 ha = __ldg(hdr + 2 * (int64_t)i), hb = __ldg(hdr + 2 * (int64_t)i + 1);
   const int s0 = ha.x, m = ha.y, np = ha.z, ns = ha.w;
   const uint32_t* L = list + ((int64_t)(uint32_t)hb.x | ((int64_t)hb.y << 32));
-  uint32_t next = tid < np ? __ldg(L + tid) : 0u;
   stage_basis<float, 12, 4>(Us, U, rot, sup_idx, s0, m, tid, kThreads);
   for (int s = tid; s < m; s += kThreads) rows[s] = __ldg(sup_row + s0 + s);
   if (tid == 0) rows[m] = make_int2(hb.z, hb.w);
@@ -930,76 +945,83 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) k_couple_pairs(
   if (tid < 9) out[18 + tid] = __ldg(bsr + block_row_at<float>(hb.z, hb.w, 0, tid / 3) + tid % 3);
   __syncthreads();
 
-  float M[9], A[9], b[3] = {0, 0, 0};
-  mat3_zero(M);
-  mat3_zero(A);
-  for (int r = tid; r < m; r += kThreads) {
-    float H[9], Uj[9], T[9], g0, g1, g2;
-    const int j = __ldg(sup_idx + s0 + r);
-    load_slot(Us + 12 * r, Uj);
-    if (diag_g) {
-      const float4 a = diag_g[3 * (int64_t)j], h = diag_g[3 * (int64_t)j + 1], c = diag_g[3 * (int64_t)j + 2];
-      H[0] = a.x; H[1] = H[3] = a.y; H[2] = H[6] = a.z; H[4] = a.w; H[5] = H[7] = h.x; H[8] = h.y;
-      g0 = h.z; g1 = h.w; g2 = c.x;
-    } else {
-      const int2 row = rows[r];
-      load_block(bsr, row.x, row.y, 0, H);
-      g0 = g_hi[3 * (int64_t)j];
-      g1 = g_hi[3 * (int64_t)j + 1];
-      g2 = g_hi[3 * (int64_t)j + 2];
+  float sum[3] = {0, 0, 0};
+#pragma unroll 1
+  for (int share = 0; share < kShares; ++share) {
+    const int vt = tid + kThreads * share;
+    uint32_t next = vt < np ? __ldg(L + vt) : 0u;
+    float M[9], A[9], b[3] = {0, 0, 0};
+    mat3_zero(M);
+    mat3_zero(A);
+    for (int r = vt; r < m; r += kStep) {
+      float H[9], Uj[9], T[9], g0, g1, g2;
+      const int j = __ldg(sup_idx + s0 + r);
+      load_slot(Us + 12 * r, Uj);
+      if (diag_g) {
+        const float4 a = diag_g[3 * (int64_t)j], h = diag_g[3 * (int64_t)j + 1], c = diag_g[3 * (int64_t)j + 2];
+        H[0] = a.x; H[1] = H[3] = a.y; H[2] = H[6] = a.z; H[4] = a.w; H[5] = H[7] = h.x; H[8] = h.y;
+        g0 = h.z; g1 = h.w; g2 = c.x;
+      } else {
+        const int2 row = rows[r];
+        load_block(bsr, row.x, row.y, 0, H);
+        g0 = g_hi[3 * (int64_t)j];
+        g1 = g_hi[3 * (int64_t)j + 1];
+        g2 = g_hi[3 * (int64_t)j + 2];
+      }
+      mat3_zero(T);
+      mat3_mul_acc(H, Uj, T);
+#pragma unroll
+      for (int c = 0; c < 9; ++c) T[c] *= 0.5f;
+      mat3_tmul_acc(Uj, T, M);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) b[c] += Uj[c] * g0 + Uj[3 + c] * g1 + Uj[6 + c] * g2;
     }
-    mat3_zero(T);
-    mat3_mul_acc(H, Uj, T);
-#pragma unroll
-    for (int c = 0; c < 9; ++c) T[c] *= 0.5f;
-    mat3_tmul_acc(Uj, T, M);
-#pragma unroll
-    for (int c = 0; c < 3; ++c) b[c] += Uj[c] * g0 + Uj[3 + c] * g1 + Uj[6 + c] * g2;
-  }
-  for (int e = tid; e < np; e += kThreads) {
-    const uint32_t w = next;
-    if (e + kThreads < np) next = __ldg(L + e + kThreads);
-    const int r = w & 1023, l = (w >> 10) & 1023;
-    float H[9], Ul[9], Uj[9], T[9];
-    const int2 row = rows[r];
-    load_block(bsr, row.x, row.y, (int)(w >> 20), H);
-    load_slot(Us + 12 * l, Ul);
-    mat3_zero(T);
-    mat3_mul_acc(H, Ul, T);
-    load_slot(Us + 12 * r, Uj);
-    mat3_tmul_acc(Uj, T, M);
-  }
-  if (kUpd == CC_UPDATE_CC) {
-    for (int e = tid ^ (kThreads / 2); e < ns; e += kThreads) {
-      const uint32_t w = __ldg(L + np + e);
+    for (int e = vt; e < np; e += kStep) {
+      const uint32_t w = next;
+      if (e + kStep < np) next = __ldg(L + e + kStep);
       const int r = w & 1023, l = (w >> 10) & 1023;
-      const bool lower = l == (int)kPairSelf;  // stored as H_ji, j = row r of the support
-      float H[9], Uv[9];
+      float H[9], Ul[9], Uj[9], T[9];
       const int2 row = rows[r];
       load_block(bsr, row.x, row.y, (int)(w >> 20), H);
-      load_slot(Us + 12 * (lower ? r : l), Uv);
-      if (lower) {
-        float t;
-        t = H[1]; H[1] = H[3]; H[3] = t;
-        t = H[2]; H[2] = H[6]; H[6] = t;
-        t = H[5]; H[5] = H[7]; H[7] = t;
-      }
-      mat3_mul_acc(H, Uv, A);
+      load_slot(Us + 12 * l, Ul);
+      mat3_zero(T);
+      mat3_mul_acc(H, Ul, T);
+      load_slot(Us + 12 * r, Uj);
+      mat3_tmul_acc(Uj, T, M);
     }
-  }
+    if (kUpd == CC_UPDATE_CC) {
+      for (int e = vt ^ (kStep / 2); e < ns; e += kStep) {
+        const uint32_t w = __ldg(L + np + e);
+        const int r = w & 1023, l = (w >> 10) & 1023;
+        const bool lower = l == (int)kPairSelf;  // stored as H_ji, j = row r of the support
+        float H[9], Uv[9];
+        const int2 row = rows[r];
+        load_block(bsr, row.x, row.y, (int)(w >> 20), H);
+        load_slot(Us + 12 * (lower ? r : l), Uv);
+        if (lower) {
+          float t;
+          t = H[1]; H[1] = H[3]; H[3] = t;
+          t = H[2]; H[2] = H[6]; H[6] = t;
+          t = H[5]; H[5] = H[7]; H[7] = t;
+        }
+        mat3_mul_acc(H, Uv, A);
+      }
+    }
 
-  reduce18<float, kWarps>(M, A, b, red, out);
+    reduce18<float, kWarps, kShares == 2>(M, A, b, red, out, sum, share);
+  }
   if constexpr (kFuse) condense_group_tail<double, float, true, kUpd>(ca, 1e-12);
 }
 
-template <int kThreads, int kUpd>
+template <int kThreads, int kUpd, int kShares = 1>
 void launch_couple_pairs(Mesh& m, const int32_t* verts, int64_t count, const float* U, const float* bsr,
                          const float* g_hi, float* cpl, const float* rot, const CondenseArgs<float>& ca, bool fuse,
                          cudaStream_t s) {
   const int supm = m.sup_max > 0 ? m.sup_max : 1;
   const size_t smem = align16((size_t)supm * 12 * sizeof(float)) + (size_t)(supm + 1) * sizeof(int2);
   // the limit on supports is the one of the slot-map kernels, whichever kernel runs
-  CCG_CHECK(kThreads == 32 || cta_smem_bytes<float>(supm, m.smap_max, m.smap_wide ? 2 : 1, kThreads) <= 220 * 1024,
+  constexpr int kDealt = kThreads * kShares;
+  CCG_CHECK(kDealt == 32 || cta_smem_bytes<float>(supm, m.smap_max, m.smap_wide ? 2 : 1, kDealt) <= 220 * 1024,
             CC_ERR_INVALID_ARG, "support too large for the coupling kernel");
   auto go = [&](auto kern) {
     set_smem_limit(reinterpret_cast<const void*>(kern), smem);
@@ -1007,8 +1029,8 @@ void launch_couple_pairs(Mesh& m, const int32_t* verts, int64_t count, const flo
                (const int32_t*)m.d_sup_idx.p, (const int2*)m.d_sup_row.p, U, (const uint32_t*)m.d_pairs.p, bsr,
                g_hi, rows_from_positions(m, true) ? (const float4*)m.mx.diag_g.p : nullptr, supm, rot, cpl, ca);
   };
-  if (fuse) go(k_couple_pairs<kThreads, kUpd, true>);
-  else go(k_couple_pairs<kThreads, kUpd, false>);
+  if (fuse) go(k_couple_pairs<kThreads, kUpd, true, kShares>);
+  else go(k_couple_pairs<kThreads, kUpd, false, kShares>);
   CCG_CUDA(cudaGetLastError());
 }
 
@@ -1142,6 +1164,14 @@ void launch_couple_rows64(Mesh& m, const int32_t* verts, int64_t count, const do
   CCG_CUDA(cudaGetLastError());
 }
 
+// Colours of more vertices than an SM's 32 CTAs hold on the chip's 152 SMs take
+// one warp a vertex instead of two (two shares, the same bits): no barrier, and
+// the last warp's wait for its loads is no longer the first's.  Below that the
+// two warps' shorter chain counts.  Mixed sweep of the 64^3 cube (66 000 vertices
+// a colour) 1.85 -> 1.74 ms, of the 32^3 cube (8 440) 368 -> 359 us; restarted
+// 16^3 solve (1 084) 2.45 -> 2.51 ms, 8^3 sweep (142) 143 -> 155 us.
+constexpr int64_t kCoupleOneWarpMin = 152 * 32;
+
 template <typename HT, bool kMixed, int kUpd>
 void launch_one(Mesh& m, const int32_t* verts, int64_t count, const HT* U, const HT* bsr, const double* g64,
                 const float* g_hi, const float* g_lo, HT* cpl, double* x, SweepCounters c, cudaStream_t s) {
@@ -1166,7 +1196,12 @@ void launch_one(Mesh& m, const int32_t* verts, int64_t count, const HT* U, const
         done = true;
         switch (m.tune_couple_threads) {
           case 32: launch_couple_pairs<32, kUpd>(m, verts, count, U, bsr, g_hi, cpl, rot, cf, fuse, s); break;
-          case 64: launch_couple_pairs<64, kUpd>(m, verts, count, U, bsr, g_hi, cpl, rot, cf, fuse, s); break;
+          case 64:
+            if (!fuse && count > kCoupleOneWarpMin)
+              launch_couple_pairs<32, kUpd, 2>(m, verts, count, U, bsr, g_hi, cpl, rot, cf, false, s);
+            else
+              launch_couple_pairs<64, kUpd>(m, verts, count, U, bsr, g_hi, cpl, rot, cf, fuse, s);
+            break;
           case 256: launch_couple_pairs<256, kUpd>(m, verts, count, U, bsr, g_hi, cpl, rot, cf, fuse, s); break;
           default: launch_couple_pairs<128, kUpd>(m, verts, count, U, bsr, g_hi, cpl, rot, cf, fuse, s);
         }
