@@ -286,11 +286,16 @@ __device__ __forceinline__ bool polar_newton(const T* F, T* R) {
 // and two corrections R <- R (I + X) bring it to float64 (see polar_refine_df
 // for X).  What cancels, R^T F and R^T R - I, is formed in float64; X, about
 // 1e-7 in the first correction and 1e-14 in the second, needs only float32
-// digits of its own.  A second X above 1e-9 (a nearly singular F) leaves it to
-// the float64 iteration, about 280 float64 instructions a step against 75 a
-// correction (energy of 22 000 tets: 66 us with it).  With the sums of
-// fcr_hess_blocks in registers, three line-searched sweeps of a twisted bar:
-// 2.21 -> 1.94 ms.
+// digits of its own.  Either way the error is rounding over the smallest sum of
+// two singular values (K's smallest eigenvalue), with a larger factor here: on
+// 60 000 deformations a size, rms against 128 bits, 0.9e-16 here and 1.6e-16 by
+// the float64 iteration at singular values near 1, equal near (1, 0.1, 0.1),
+// 1.3e-15 and 0.5e-15 near (1, 0.01, 0.01).  So needles, det K below a fifth of
+// tr(S)^3 (at (1, 0.19, 0.19); one small singular value alone gives 0.25), take
+// the float64 iteration, and so does a second X above 1e-9: about 280 float64
+// instructions a step against 75 a correction (energy of 22 000 tets: 66 us
+// with it).  With the sums of fcr_hess_blocks in registers, three line-searched
+// sweeps of a twisted bar: 2.21 -> 1.94 ms.
 __device__ __forceinline__ bool polar_f64(const double* F, double* R) {
   const double det = F[0] * (F[4] * F[8] - F[5] * F[7]) + F[1] * (F[5] * F[6] - F[3] * F[8]) +
                      F[2] * (F[3] * F[7] - F[4] * F[6]);
@@ -298,12 +303,12 @@ __device__ __forceinline__ bool polar_f64(const double* F, double* R) {
   float Ff[9], R32[9];
 #pragma unroll
   for (int q = 0; q < 9; ++q) Ff[q] = (float)F[q];
-  if (!polar_newton<float>(Ff, R32)) return polar_newton<double>(F, R);
+  const bool started = polar_newton<float>(Ff, R32);
 #pragma unroll
   for (int q = 0; q < 9; ++q) R[q] = (double)R32[q];
-  float size = 0.0f;
+  float size = 0.0f, shape = 0.0f;  // of the last X; det K / tr(S)^3
 #pragma unroll 1
-  for (int it = 0; it < 2; ++it) {
+  for (int it = 0; started && it < 2; ++it) {
     double S0[9];
     float S[9], D[9], Rf[9];
 #pragma unroll
@@ -338,7 +343,7 @@ __device__ __forceinline__ bool polar_f64(const double* F, double* R) {
     K[0] += tr;
     K[4] += tr;
     K[8] += tr;
-    inv3t(K, Ki);
+    shape = inv3t(K, Ki) / (tr * tr * tr);
 #pragma unroll
     for (int r = 0; r < 3; ++r) w[r] = Ki[3 * r] * rhs[0] + Ki[3 * r + 1] * rhs[1] + Ki[3 * r + 2] * rhs[2];
     const float X[9] = {-0.5f * D[0], -0.5f * D[1] - w[2], -0.5f * D[2] + w[1],
@@ -353,7 +358,7 @@ __device__ __forceinline__ bool polar_f64(const double* F, double* R) {
       for (int c = 0; c < 3; ++c)
         R[3 * r + c] += (double)(Rf[3 * r] * X[c] + Rf[3 * r + 1] * X[3 + c] + Rf[3 * r + 2] * X[6 + c]);
   }
-  if (!(size <= 1e-9f)) return polar_newton<double>(F, R);  // also when it is NaN
+  if (!(shape >= 0.2f && size <= 1e-9f)) return polar_newton<double>(F, R);  // also when they are NaN
   return true;
 }
 
