@@ -469,7 +469,9 @@ cc_status cc_set_launch_shape(cc_mesh* mesh, int32_t couple_threads, int32_t gat
  * 1 sets, 0 clears, -1 keeps a switch; anything else is CC_ERR_INVALID_ARG.
  * Defaults: rows_from_positions 1 (measured fastest), but 0 for the mixed
  * path of a dynamic mesh (h > 0), whose steps keep the gather's float32
- * rounding (v = dx / h shows it); fused_condense 0 (measured fastest).
+ * rounding (v = dx / h shows it), and for the float64 path of a mesh with a
+ * vertex of more than about 55 tets (the gather is faster there);
+ * fused_condense 0 (measured fastest).
  * cc_autotune tries every applicable combination.  The fused and separate
  * condensations give identical results; the two row builds agree within the
  * rounding of the path's precision. */

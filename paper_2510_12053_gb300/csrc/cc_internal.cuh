@@ -276,6 +276,7 @@ struct Mesh {
   DBuf<uint32_t> d_pairs;
   // rows formed from the positions (kernels_rows.cu; stable Neo-Hookean)
   bool rows_ok = false;      // the mesh fits that kernel (build_row_data)
+  bool rows64_fast = false;  // and its float64 rows leave an SM enough warps (kRows64FastSmem)
   int32_t max_ring = 0;      // most 1-ring neighbours of a vertex
   float len_scale = 1.0f;    // power of two that brings the mean edge near 1 (mixed path)
   DBuf<int4> d_row_hdr2;     // [2 n_free] (j, first upper block, upper blocks, first ring entry),
@@ -331,6 +332,15 @@ bool pdl_enabled();  // true when CC_GB300_PDL is set in the environment (defaul
 
 // Shared memory one CTA of the row kernel may take.
 constexpr size_t kRowsSmemMax = 200 * 1024;
+// Most shared memory a warp of the float64 row kernel may take by default: it
+// is sized by the mesh's largest valence, so one vertex of many tets costs every
+// row its warps, which the gather does not notice.  A refresh of a box with one
+// vertex of V tets, store + gather against positions, 24^3 cells: V = 24 123 / 68
+// us, 48 136 / 121, 64 143 / 136, 80 151 / 225, 200 206 / 483; 8^3 cells: 24 48 /
+// 19, 48 59 / 53, 64 63 / 68, 200 109 / 193.  40 KB is a vertex of 53 to 56 tets.
+// The mixed kernel takes a quarter of that and is faster at every valence up to
+// 240 (32^3 cells: 66 / 31 us at 24, 148 / 112 at 240).
+constexpr size_t kRows64FastSmem = 40 * 1024;
 
 // Stable Neo-Hookean block rows are formed from the positions instead of a
 // per-tet Hessian store (kernels_rows.cu); Fixed Corotational keeps the store
@@ -350,7 +360,8 @@ inline bool fused_local_solve(const Mesh& m, cc_update upd) {
 inline bool mixed_dynamic(const Mesh& m, bool mixed) { return mixed && m.h > 0.0; }
 
 inline bool rows_from_positions(const Mesh& m, bool mixed) {
-  return m.rows_ok && (m.rows_build < 0 ? !mixed_dynamic(m, mixed) : m.rows_build != 0);
+  const bool by_default = mixed ? !mixed_dynamic(m, mixed) : m.rows64_fast;
+  return m.rows_ok && (m.rows_build < 0 ? by_default : m.rows_build != 0);
 }
 
 // The float64 Hessian that bases are built from: a dynamic mesh's keeps the

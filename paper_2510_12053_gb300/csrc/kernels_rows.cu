@@ -582,7 +582,7 @@ void launch_rows_from_positions(Mesh& m, bool mixed, const double* x, const doub
 // on the device from the uploaded topology.  Sets rows_ok: the ring slots fit
 // a byte and one warp's four rows fit the shared memory in both precisions.
 void build_row_data(Mesh& m, const std::vector<double>& volw) {
-  m.rows_ok = false;
+  m.rows_ok = m.rows64_fast = false;
   if (m.model != CC_MODEL_SNH) return;
   m.max_ring = 0;
   for (int64_t v = 0; v < m.n; ++v)
@@ -645,6 +645,7 @@ void build_row_data(Mesh& m, const std::vector<double>& volw) {
   CCG_CUDA(cudaGetLastError());
   CCG_CUDA(cudaStreamSynchronize(s));  // host vectors above go out of scope
   m.rows_ok = true;
+  m.rows64_fast = rows_f64_smem(m.max_valence, m.max_ring) <= kRows64FastSmem;
 }
 
 }  // namespace ccg
