@@ -55,7 +55,9 @@ void drop_graph(Mesh& m) {
   m.prof.graph_launches = 0;
 }
 
-void ensure_state(Mesh& m, cc_precision p) {
+// A group of buffers counts as there once its last one is: a group that ran out
+// of memory half-way is allocated again by the next call.
+static void alloc_state(Mesh& m, cc_precision p) {
   cudaStream_t s = m.stream;
   const size_t ne = 4 * (size_t)m.T;
   if (!m.d_grp_cnt.p) {  // arrival counters of the fused local solves (they reset themselves)
@@ -68,14 +70,14 @@ void ensure_state(Mesh& m, cc_precision p) {
       m.f64.gcon.alloc(3 * ne);
       m.f64.hten.alloc(kTetStore * (size_t)m.T);
     }
-    if (!m.f64.g.p) {
+    if (!state_allocated(m, p)) {
       m.f64.g.alloc(3 * m.n);
       m.f64.bsr.alloc(12 * m.nnz_up);
       m.f64.cpl.alloc(32 * m.n_free);
       CCG_CUDA(cudaMemsetAsync(m.f64.g.p, 0, 3 * m.n * sizeof(double), s));
     }
   } else {
-    if (!m.mx.g_hi.p) {
+    if (!state_allocated(m, p)) {
       m.mx.g_hi.alloc(3 * m.n);
       m.mx.g_lo.alloc(3 * m.n);
       m.mx.bsr.alloc(12 * m.nnz_up);
@@ -101,6 +103,14 @@ void ensure_state(Mesh& m, cc_precision p) {
       m.mx.hten.alloc(kTetStore * (size_t)m.T);
     }
   }
+}
+
+bool state_allocated(const Mesh& m, cc_precision p) {
+  return p == CC_PREC_FP64 ? m.f64.cpl.p != nullptr : m.mx.xt_lo.p != nullptr;
+}
+
+void ensure_state(Mesh& m, cc_precision p) {
+  with_room(m, [&] { alloc_state(m, p); });
 }
 
 namespace {
@@ -287,6 +297,11 @@ void check_sweep_opts(const Mesh& m, const cc_sweep_opts& o, int* cb, int* ce) {
   }
 }
 
+// State and lists that sweeps of these options read.
+void prepare_sweeps(Mesh& m, const cc_sweep_opts& o) {
+  ensure_state(m, o.precision);
+  if (o.update != CC_UPDATE_CD) ensure_coupling_lists(m, o.precision == CC_PREC_MIXED);
+}
 
 // Every mesh of a batch takes part again (cc_solve_batch may have stopped some).
 void activate_all(Mesh& m) {
@@ -496,23 +511,26 @@ cc_status cc_set_subspace(cc_mesh* m, const int64_t* sup_ptr, const int32_t* sup
     const int64_t total = sup_ptr[n];
     CCG_CHECK(total < (int64_t(1) << 31) && supmax < 32768, CC_ERR_INVALID_ARG, "support too large");
     drop_graph(*m);
+    const int32_t ring = m->k_ring == 0 ? -1 : m->k_ring;  // -1: custom
+    m->k_ring = 0;  // no subspace until the new one is in place
     m->sup_ptr.assign(sup_ptr, sup_ptr + n + 1);
     m->sup_idx.assign(sup_idx, sup_idx + total);
     m->sup_max = supmax;
     int hs = 32;
     while (hs < 2 * std::max(supmax, 1)) hs <<= 1;
     m->hash_size = hs;
-    if (m->k_ring == 0) m->k_ring = -1;  // custom
+    reset_coupling_lists(*m);
     std::vector<int32_t> sp32(n + 1);
     for (int64_t v = 0; v <= n; ++v) sp32[v] = (int32_t)sup_ptr[v];
     m->d_sup_ptr.upload(sp32, m->stream);
     m->d_sup_idx.upload(m->sup_idx, m->stream);
-    ccg::build_slot_maps(*m);
     m->f64.U.alloc(9 * std::max<int64_t>(total, 1));
     if (total) CCG_CUDA(cudaMemcpyAsync(m->f64.U.p, U, 9 * total * sizeof(double), cudaMemcpyHostToDevice, m->stream));
     m->mx.U.alloc(9 * std::max<int64_t>(total, 1));
     ccg::bases_to_f32(*m);
     CCG_CUDA(cudaStreamSynchronize(m->stream));
+    m->k_ring = ring;
+    ensure_coupling_lists(*m, true);
   })
 }
 
@@ -546,7 +564,7 @@ cc_status cc_sweep(cc_mesh* m, double* x, const double* xt, const cc_sweep_opts*
     CCG_CHECK(m->h == 0.0 || xt, CC_ERR_INVALID_ARG, "dynamic mesh needs xtilde");
     int cb, ce;
     check_sweep_opts(*m, *opts, &cb, &ce);
-    ensure_state(*m, opts->precision);
+    prepare_sweeps(*m, *opts);
     cudaStream_t s = m->stream;
     CCG_CUDA(cudaMemsetAsync(m->d_counters.p, 0, 8 * sizeof(unsigned long long), s));
     activate_all(*m);
@@ -572,16 +590,17 @@ cc_status cc_solve_step(cc_mesh* m, double* x, double* v, const cc_step_opts* o,
     cc_sweep_opts so{o->update, o->schedule, o->precision, 0, -1, o->corotated};
     int cb, ce;
     check_sweep_opts(*m, so, &cb, &ce);
-    ensure_state(*m, o->precision);
+    prepare_sweeps(*m, so);
     cudaStream_t s = m->stream;
     const int64_t n = m->n;
     const bool dyn = m->h > 0.0;
     const double* xt = nullptr;
     if (dyn) {
-      if (!m->d_xtilde.p) {
-        m->d_xtilde.alloc(3 * n);
-        m->d_xold.alloc(3 * n);
-      }
+      if (!m->d_xold.p)
+        with_room(*m, [&] {
+          m->d_xtilde.alloc(3 * n);
+          m->d_xold.alloc(3 * n);
+        });
       CCG_CUDA(cudaMemcpyAsync(m->d_xold.p, x, 3 * n * sizeof(double), cudaMemcpyDeviceToDevice, s));
       const int e0 = prof_event(*m);
       launch_inertial_target(x, v, n, m->h, m->grav, m->d_xtilde.p, s);
@@ -644,10 +663,11 @@ cc_status cc_solve_step(cc_mesh* m, double* x, double* v, const cc_step_opts* o,
     // Global backtracking line search (Sec. 4.4): the sweep's displacement is
     // the direction, the step the largest 2^-k (k < 30) that does not raise E.
     if (o->line_search && !conv && it < o->max_iters) {
-      if (!m->d_xls0.p) {
-        m->d_xls0.alloc(3 * n);
-        m->d_xls1.alloc(3 * n);
-      }
+      if (!m->d_xls1.p)
+        with_room(*m, [&] {
+          m->d_xls0.alloc(3 * n);
+          m->d_xls1.alloc(3 * n);
+        });
       auto energy_at = [&](const double* xe) {
         const int ee = prof_event(*m);
         launch_energy(*m, xe, xt, m->d_scalars.p + 1, s);
@@ -826,17 +846,18 @@ cc_status cc_solve_batch(cc_mesh* m, double* x, double* v, const cc_step_opts* o
     cc_sweep_opts so{o->update, o->schedule, o->precision, 0, -1, o->corotated};
     int cb, ce;
     check_sweep_opts(*m, so, &cb, &ce);
-    ensure_state(*m, o->precision);
+    prepare_sweeps(*m, so);
     cudaStream_t s = m->stream;
     const int64_t n = m->n;
     const int32_t B = (int32_t)m->mesh_vptr.size() - 1;
     const bool dyn = m->h > 0.0;
     const double* xt = nullptr;
     if (dyn) {
-      if (!m->d_xtilde.p) {
-        m->d_xtilde.alloc(3 * n);
-        m->d_xold.alloc(3 * n);
-      }
+      if (!m->d_xold.p)
+        with_room(*m, [&] {
+          m->d_xtilde.alloc(3 * n);
+          m->d_xold.alloc(3 * n);
+        });
       CCG_CUDA(cudaMemcpyAsync(m->d_xold.p, x, 3 * n * sizeof(double), cudaMemcpyDeviceToDevice, s));
       launch_inertial_target(x, v, n, m->h, m->grav, m->d_xtilde.p, s);
       xt = m->d_xtilde.p;
@@ -924,10 +945,11 @@ cc_status cc_solve_batch(cc_mesh* m, double* x, double* v, const cc_step_opts* o
     // the largest 2^-k (k < 30) of its own sweep displacement that does not
     // raise its own energy, 0 if none; every trial is one launch for all.
     if (o->line_search && live > 0 && it < o->max_iters) {
-      if (!m->d_xls0.p) {
-        m->d_xls0.alloc(3 * n);
-        m->d_xls1.alloc(3 * n);
-      }
+      if (!m->d_xls1.p)
+        with_room(*m, [&] {
+          m->d_xls0.alloc(3 * n);
+          m->d_xls1.alloc(3 * n);
+        });
       std::vector<double> E0(B), E1(B), alpha(B);
       std::vector<char> searching(B);
       auto energies = [&](const double* xe, std::vector<double>& out) {
@@ -1100,10 +1122,10 @@ cc_status cc_autotune(cc_mesh* m, const double* x, const double* xt, cc_precisio
     cc_sweep_opts so{CC_UPDATE_CC, CC_SCHED_COLORED, p, 0, -1};
     int cb, ce;
     check_sweep_opts(*m, so, &cb, &ce);
-    ensure_state(*m, p);
+    prepare_sweeps(*m, so);
     cudaStream_t s = m->stream;
     DBuf<double> tmp;
-    tmp.alloc(3 * m->n);
+    with_room(*m, [&] { tmp.alloc(3 * m->n); });
     cudaEvent_t e0, e1;
     CCG_CUDA(cudaEventCreate(&e0));
     CCG_CUDA(cudaEventCreate(&e1));
@@ -1235,8 +1257,8 @@ cc_status cc_set_sweep_variant(cc_mesh* m, int32_t rows_from_positions, int32_t 
     if (fused_condense >= 0) m->fused_condense = fused_condense != 0;
     drop_graph(*m);
     // what the chosen row build needs (the per-tet store or the per-tet sigma)
-    if (m->mx.g_hi.p) ensure_state(*m, CC_PREC_MIXED);
-    if (m->f64.g.p) ensure_state(*m, CC_PREC_FP64);
+    if (state_allocated(*m, CC_PREC_MIXED)) ensure_state(*m, CC_PREC_MIXED);
+    if (state_allocated(*m, CC_PREC_FP64)) ensure_state(*m, CC_PREC_FP64);
   })
 }
 

@@ -219,7 +219,7 @@ struct Mesh {
   int32_t k_ring = 0;
   int32_t sup_max = 0;
   int32_t hash_size = 0;       // unused (kept for layout stability)
-  int64_t smap_max = 0;        // longest per-vertex slot map
+  int64_t smap_max = 0;        // longest per-vertex slot map (whether or not the maps exist)
   bool smap_wide = false;      // slot maps in uint16 (supports of 250+ vertices)
 
   // device rest data
@@ -261,16 +261,17 @@ struct Mesh {
   // block of each support row and of row i (in support order, row i last):
   // the block column's slot in S_i, or kSlotNone / kSlotSelf (column i) /
   // kSlotDiag (the row's diagonal block).
+  bool smap_ok = false;      // the maps of the current supports exist (ensure_coupling_lists)
   DBuf<int64_t> d_smap_ptr;  // [n+1]
   DBuf<uint8_t> d_smap8;
   DBuf<uint16_t> d_smap16;
-  // Pair lists of the float32 coupling kernel (k_couple_pairs): for free vertex
-  // i, the blocks (j, l), j < l, of the support's upper rows, then the ns
+  // Pair lists of the other coupling kernels (k_couple_pairs, k_couple_rows64):
+  // for free vertex i, the blocks (j, l), j < l, of the support's upper rows, then the ns
   // blocks that couple a support row with i.  An entry is
   // row slot | column slot << 10 | place in the row << 20; the slot of i is
   // |S_i|, and kPairSelf as column slot marks a block (j, i) of a support row.
   // Empty when a support or a row does not fit the fields.
-  bool pairs_ok = false;
+  bool pairs_ok = false, pairs_tried = false;
   DBuf<int4> d_pair_hdr;       // [2n] (first support entry, |S_i|, pairs, ns), (list start lo, hi, first block of row i, blocks)
   DBuf<int2> d_sup_row;        // [support_total] first upper block and blocks of every support vertex's row
   DBuf<uint32_t> d_pairs;
@@ -359,6 +360,8 @@ inline bool fused_local_solve(const Mesh& m, cc_update upd) {
 // they have always had, and a step its bits.
 inline bool mixed_dynamic(const Mesh& m, bool mixed) { return mixed && m.h > 0.0; }
 
+inline bool couples_from_pairs(const Mesh& m, bool mixed) { return !mixed_dynamic(m, mixed); }
+
 inline bool rows_from_positions(const Mesh& m, bool mixed) {
   const bool by_default = mixed ? !mixed_dynamic(m, mixed) : m.rows64_fast;
   return m.rows_ok && (m.rows_build < 0 ? by_default : m.rows_build != 0);
@@ -387,9 +390,29 @@ void pdl_launch(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cuda
 // Host-side helpers implemented in mesh_build.cpp (topology, plain C++)
 // ---------------------------------------------------------------------------
 void build_topology(Mesh& m);
-// Slot maps for the current supports (after cc_build_subspace / cc_set_subspace;
-// kernels_setup.cu, built on the device: d_sup_ptr / d_sup_idx must be uploaded).
-void build_slot_maps(Mesh& m);
+// What the coupling kernel of a precision reads, for the current supports
+// (kernels_setup.cu, built on the device: d_sup_ptr / d_sup_idx must be
+// uploaded): the pair lists, or the slot maps where those are not used, do not
+// fit their fields or found no memory.  Built once per subspace and kernel: at
+// the end of a set-up call for the mixed path, which a float64 sweep of a static
+// mesh shares; for a float64 sweep of a dynamic mesh before the first one.
+void ensure_coupling_lists(Mesh& m, bool mixed);
+// Called when the supports change, with m.sup_* in place.
+void reset_coupling_lists(Mesh& m);
+// Gives the pair lists' memory back (the slot maps, smaller, take their place);
+// false when there are none.
+bool drop_pair_lists(Mesh& m);
+// Runs f, which allocates.  The pair lists are only the faster way: where f
+// finds no memory beside them it runs again without them.
+template <typename F>
+void with_room(Mesh& m, F&& f) {
+  try {
+    f();
+  } catch (const Fail& e) {
+    if (e.st != CC_ERR_OOM || !drop_pair_lists(m)) throw;
+    f();
+  }
+}
 // host worker threads for setup passes, and a parallel loop over vertex ranges
 int host_threads(int64_t items);
 void parallel_ranges(int64_t n, int nt, const std::function<void(int, int64_t, int64_t)>& f);
@@ -467,6 +490,7 @@ int64_t patch_solves_shared(Mesh& m, const int32_t* d_verts, int64_t count, bool
 void bases_to_f32(Mesh& m);
 // solver state of one precision (allocated once, on first use)
 void ensure_state(Mesh& m, cc_precision p);
+bool state_allocated(const Mesh& m, cc_precision p);
 // forgets the captured sweep graph (its nodes hold buffer pointers)
 void drop_graph(Mesh& m);
 void clear_error();

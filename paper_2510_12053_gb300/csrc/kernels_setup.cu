@@ -242,8 +242,6 @@ void build_color_lists(Mesh& m) {
   CCG_CUDA(cudaStreamSynchronize(s));
 }
 
-// k-ring supports on the host: breadth-first over the 1-ring CSR, free
-// vertices only, i excluded, ascending.  Uploads them and the slot maps.
 namespace {
 // Index of key in the ascending a[0..m), or -1.
 __device__ __forceinline__ int find_in_sorted(const int32_t* __restrict__ a, int m, int key) {
@@ -381,63 +379,56 @@ __global__ void k_pair_lists(const int32_t* __restrict__ rows, int64_t nrows, co
 }  // namespace
 
 // Pair lists of the current supports; the host places the vertices' lists.
+// Without memory for them pairs_ok stays false.
 static void build_pair_lists(Mesh& m) {
   cudaStream_t s = m.stream;
-  m.pairs_ok = false;
-  m.d_pairs.release();
+  m.pairs_tried = true;
   if (m.sup_max > kPairMaxSup || m.max_up > kPairMaxRow || m.n_free <= 0) return;
   const int64_t nf = m.n_free, total = m.sup_ptr[m.n];
   const unsigned grid = (unsigned)((nf * 32 + 255) / 256);
-  DBuf<int2> d_counts;
-  d_counts.alloc(nf);
-  k_pair_lists<false><<<grid, 256, 0, s>>>(m.d_free_rows.p, nf, m.d_sup_ptr.p, m.d_sup_idx.p, m.d_up_ptr.p,
-                                           m.d_up_col.p, d_counts.p, nullptr, nullptr, nullptr);
-  std::vector<int2> counts(nf);
-  CCG_CUDA(cudaMemcpyAsync(counts.data(), d_counts.p, nf * sizeof(int2), cudaMemcpyDeviceToHost, s));
-  CCG_CUDA(cudaStreamSynchronize(s));
-  std::vector<int4> hdr(2 * m.n, make_int4(0, 0, 0, 0));
-  int64_t at = 0, w = 0;
-  for (int64_t v = 0; v < m.n; ++v) {
-    if (m.pinned[v]) continue;
-    const int2 c = counts[w++];
-    hdr[2 * v] = make_int4((int)m.sup_ptr[v], (int)(m.sup_ptr[v + 1] - m.sup_ptr[v]), c.x, c.y);
-    hdr[2 * v + 1] = make_int4((int)(uint32_t)(at & 0xffffffff), (int)(at >> 32), (int)m.up_ptr[v],
-                             (int)(m.up_ptr[v + 1] - m.up_ptr[v]));
-    at += c.x + c.y;
-  }
   try {
-    m.d_pair_hdr.upload(hdr, s);
+    DBuf<int2> d_counts;
+    d_counts.alloc(nf);
+    k_pair_lists<false><<<grid, 256, 0, s>>>(m.d_free_rows.p, nf, m.d_sup_ptr.p, m.d_sup_idx.p, m.d_up_ptr.p,
+                                             m.d_up_col.p, d_counts.p, nullptr, nullptr, nullptr);
+    std::vector<int2> counts(nf);
+    CCG_CUDA(cudaMemcpyAsync(counts.data(), d_counts.p, nf * sizeof(int2), cudaMemcpyDeviceToHost, s));
+    CCG_CUDA(cudaStreamSynchronize(s));
+    std::vector<int4> hdr(2 * m.n, make_int4(0, 0, 0, 0));
+    int64_t at = 0, w = 0;
+    for (int64_t v = 0; v < m.n; ++v) {
+      if (m.pinned[v]) continue;
+      const int2 c = counts[w++];
+      hdr[2 * v] = make_int4((int)m.sup_ptr[v], (int)(m.sup_ptr[v + 1] - m.sup_ptr[v]), c.x, c.y);
+      hdr[2 * v + 1] = make_int4((int)(uint32_t)(at & 0xffffffff), (int)(at >> 32), (int)m.up_ptr[v],
+                                 (int)(m.up_ptr[v + 1] - m.up_ptr[v]));
+      at += c.x + c.y;
+    }
     m.d_sup_row.alloc(total);
     m.d_pairs.alloc(at);
-  } catch (const Fail& f) {  // no room for them: the slot-map kernels need only what follows
-    if (f.st != CC_ERR_OOM) throw;
-    cudaGetLastError();
-    clear_error();
+    m.d_pair_hdr.upload(hdr, s);
+    k_pair_lists<true><<<grid, 256, 0, s>>>(m.d_free_rows.p, nf, m.d_sup_ptr.p, m.d_sup_idx.p, m.d_up_ptr.p,
+                                            m.d_up_col.p, nullptr, m.d_pair_hdr.p, m.d_sup_row.p, m.d_pairs.p);
+    CCG_CUDA(cudaGetLastError());
+    CCG_CUDA(cudaStreamSynchronize(s));  // the host vectors above go out of scope
+    m.pairs_ok = true;
+  } catch (const Fail& f) {
     m.d_pair_hdr.release();
     m.d_sup_row.release();
     m.d_pairs.release();
-    CCG_CUDA(cudaStreamSynchronize(s));
-    return;
+    if (f.st != CC_ERR_OOM) throw;
+    cudaGetLastError();
+    clear_error();
   }
-  k_pair_lists<true><<<grid, 256, 0, s>>>(m.d_free_rows.p, nf, m.d_sup_ptr.p, m.d_sup_idx.p, m.d_up_ptr.p,
-                                          m.d_up_col.p, nullptr, m.d_pair_hdr.p, m.d_sup_row.p, m.d_pairs.p);
-  CCG_CUDA(cudaGetLastError());
-  CCG_CUDA(cudaStreamSynchronize(s));  // the host vectors above go out of scope
-  m.pairs_ok = true;
 }
 
-// Slot maps of the current supports (cc_build_subspace / cc_set_subspace),
-// built on the device from the uploaded supports and upper block pattern.
-// The host only sums the row lengths per vertex for the offsets.
-void build_slot_maps(Mesh& m) {
-  const int64_t n = m.n;
-  cudaStream_t s = m.stream;
-  build_pair_lists(m);
-  m.smap_wide = m.sup_max >= 250;
-  std::vector<int64_t> len(n, 0);
-  const int nt = host_threads(n);
+// Entries of the vertices' slot maps; the longest one also sets the limit on
+// supports (launch_couple_pairs).
+static std::vector<int64_t> slot_map_lengths(const Mesh& m, int64_t* longest) {
+  std::vector<int64_t> len(m.n, 0);
+  const int nt = host_threads(m.n);
   std::vector<int64_t> longest_t(nt, 0);
-  parallel_ranges(n, nt, [&](int t, int64_t v0, int64_t v1) {
+  parallel_ranges(m.n, nt, [&](int t, int64_t v0, int64_t v1) {
     for (int64_t v = v0; v < v1; ++v) {
       if (m.pinned[v]) continue;
       int64_t c = m.up_ptr[v + 1] - m.up_ptr[v];
@@ -449,23 +440,31 @@ void build_slot_maps(Mesh& m) {
       longest_t[t] = std::max(longest_t[t], c);
     }
   });
+  *longest = *std::max_element(longest_t.begin(), longest_t.end());
+  return len;
+}
+
+// Slot maps of the current supports, built on the device from the uploaded
+// supports and upper block pattern.  The host only sums the row lengths per
+// vertex for the offsets.
+static void build_slot_maps(Mesh& m) {
+  const int64_t n = m.n;
+  cudaStream_t s = m.stream;
+  const std::vector<int64_t> len = slot_map_lengths(m, &m.smap_max);
   std::vector<int64_t> ptr(n + 1, 0);
   for (int64_t v = 0; v < n; ++v) ptr[v + 1] = ptr[v] + len[v];
-  m.smap_max = *std::max_element(longest_t.begin(), longest_t.end());
   m.d_smap_ptr.upload(ptr, s);
 
   const int64_t total = std::max<int64_t>(ptr[n], 1);
   const unsigned grid = (unsigned)((m.n_free * 32 + 255) / 256);
   if (m.smap_wide) {
     m.d_smap16.alloc(total + kSlotMapSlack);
-    m.d_smap8.release();
     CCG_CUDA(cudaMemsetAsync(m.d_smap16.p + total, 0, kSlotMapSlack * sizeof(uint16_t), s));
     if (m.n_free > 0)
       k_slot_maps<uint16_t><<<grid, 256, 0, s>>>(m.d_free_rows.p, m.n_free, m.d_sup_ptr.p, m.d_sup_idx.p,
                                                  m.d_up_ptr.p, m.d_up_col.p, m.d_smap_ptr.p, m.d_smap16.p);
   } else {
     m.d_smap8.alloc(total + kSlotMapSlack);
-    m.d_smap16.release();
     CCG_CUDA(cudaMemsetAsync(m.d_smap8.p + total, 0, kSlotMapSlack, s));
     if (m.n_free > 0)
       k_slot_maps<uint8_t><<<grid, 256, 0, s>>>(m.d_free_rows.p, m.n_free, m.d_sup_ptr.p, m.d_sup_idx.p,
@@ -473,11 +472,47 @@ void build_slot_maps(Mesh& m) {
   }
   CCG_CUDA(cudaGetLastError());
   CCG_CUDA(cudaStreamSynchronize(s));
+  m.smap_ok = true;
 }
 
+void reset_coupling_lists(Mesh& m) {
+  m.pairs_ok = m.pairs_tried = m.smap_ok = false;
+  m.d_pair_hdr.release();
+  m.d_sup_row.release();
+  m.d_pairs.release();
+  m.d_smap_ptr.release();
+  m.d_smap8.release();
+  m.d_smap16.release();
+  m.smap_wide = m.sup_max >= 250;
+  slot_map_lengths(m, &m.smap_max);
+}
+
+void ensure_coupling_lists(Mesh& m, bool mixed) {
+  const bool pairs = couples_from_pairs(m, mixed);
+  if (pairs && !m.pairs_tried) build_pair_lists(m);
+  if (!(pairs && m.pairs_ok) && !m.smap_ok) build_slot_maps(m);
+}
+
+bool drop_pair_lists(Mesh& m) {
+  if (!m.pairs_ok) return false;
+  cudaGetLastError();
+  clear_error();
+  drop_graph(m);  // its nodes read the lists
+  m.pairs_ok = false;
+  m.d_pair_hdr.release();
+  m.d_sup_row.release();
+  m.d_pairs.release();
+  if (!m.smap_ok) build_slot_maps(m);
+  return true;
+}
+
+// k-ring supports on the host: breadth-first over the 1-ring CSR, free
+// vertices only, i excluded, ascending.  Uploads them; no subspace until the
+// bases' memory is there too.
 void build_supports(Mesh& m, int32_t k) {
   cudaStream_t s = m.stream;
   const int64_t n = m.n;
+  m.k_ring = 0;
   // vertex ranges in parallel (each with its own visit stamps); concatenated in order
   const int nt = host_threads(n);
   std::vector<std::vector<int32_t>> idx_t(nt);
@@ -522,15 +557,16 @@ void build_supports(Mesh& m, int32_t k) {
   int hs = 32;
   while (hs < 2 * std::max(supmax, 1)) hs <<= 1;
   m.hash_size = hs;
-  m.k_ring = k;
+  reset_coupling_lists(m);
   std::vector<int32_t> sp32(n + 1);
   for (int64_t v = 0; v <= n; ++v) sp32[v] = (int32_t)m.sup_ptr[v];
   m.d_sup_ptr.upload(sp32, s);
   m.d_sup_idx.upload(m.sup_idx, s);
-  build_slot_maps(m);  // on the device, from the uploaded supports
   const int64_t total = (int64_t)m.sup_idx.size();
   m.f64.U.alloc(9 * std::max<int64_t>(total, 1));
   m.mx.U.alloc(9 * std::max<int64_t>(total, 1));
+  CCG_CUDA(cudaStreamSynchronize(s));  // sp32 goes out of scope
+  m.k_ring = k;
 }
 
 // Hessian of E at x (device float64 [3][n]) in float64 into the float64
@@ -579,7 +615,7 @@ int64_t patch_solves(Mesh& m, const int32_t* d_verts, int64_t count, bool throw_
   if (3 * m.sup_max <= kPmMaxN) {
     // float32 factor + float64 refinement; the patches it hands back go to
     // the float64 kernel below
-    redo.alloc(count + 1);
+    with_room(m, [&] { redo.alloc(count + 1); });
     CCG_CUDA(cudaMemsetAsync(redo.p + count, 0, sizeof(int32_t), s));
     launch_patch_basis_mixed(m, d_verts, count, redo.p, redo.p + count, s);
     int32_t nr = 0;
@@ -595,9 +631,11 @@ int64_t patch_solves(Mesh& m, const int32_t* d_verts, int64_t count, bool throw_
   int64_t batch = std::max<int64_t>(1, (int64_t)((size_t(1) << 30) / (per * sizeof(double))));
   batch = std::min<int64_t>(batch, count);
   DBuf<double> scratch;
-  scratch.alloc(per * std::max<int64_t>(batch, 1));
   DBuf<int32_t> fail;
-  fail.alloc(1);
+  with_room(m, [&] {
+    scratch.alloc(per * std::max<int64_t>(batch, 1));
+    fail.alloc(1);
+  });
   CCG_CUDA(cudaMemsetAsync(fail.p, 0, sizeof(int32_t), s));
   for (int64_t b0 = 0; b0 < count; b0 += batch) {
     const int64_t cnt = std::min<int64_t>(batch, count - b0);
@@ -789,6 +827,7 @@ void run_subspace_build(Mesh& m, int32_t k) {
   patch_solves_shared(m, m.d_free_rows.p, m.n_free, true);
   bases_to_f32(m);
   CCG_CUDA(cudaStreamSynchronize(m.stream));
+  ensure_coupling_lists(m, true);
 }
 
 }  // namespace ccg

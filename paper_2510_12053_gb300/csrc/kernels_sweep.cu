@@ -1192,7 +1192,7 @@ void launch_one(Mesh& m, const int32_t* verts, int64_t count, const HT* U, const
     }
     bool done = false;
     if constexpr (kMixed) {
-      if (m.pairs_ok && !mixed_dynamic(m, kMixed)) {
+      if (m.pairs_ok && couples_from_pairs(m, kMixed)) {
         done = true;
         switch (m.tune_couple_threads) {
           case 32: launch_couple_pairs<32, kUpd>(m, verts, count, U, bsr, g_hi, cpl, rot, cf, fuse, s); break;
@@ -1334,15 +1334,15 @@ void launch_rotations(Mesh& m, const double* x, bool mixed, cudaStream_t s) {
     std::vector<double> soa(3 * m.n);
     for (int64_t j = 0; j < m.n; ++j)
       for (int a = 0; a < 3; ++a) soa[a * m.n + j] = m.X[3 * j + a];
-    m.d_Xrest.upload(soa, s);
+    with_room(m, [&] { m.d_Xrest.upload(soa, s); });
   }
   const unsigned grid = (unsigned)((m.n + 127) / 128);
   if (mixed) {
-    if (!m.mx.rot.p) m.mx.rot.alloc(9 * m.n);
+    if (!m.mx.rot.p) with_room(m, [&] { m.mx.rot.alloc(9 * m.n); });
     pdl_launch(k_rotations<float>, grid, 128, 0, s, m.n, (const int32_t*)m.d_nbr_ptr.p, (const int32_t*)m.d_nbr_idx.p,
                x, (const double*)m.d_Xrest.p, m.mx.rot.p);
   } else {
-    if (!m.f64.rot.p) m.f64.rot.alloc(9 * m.n);
+    if (!m.f64.rot.p) with_room(m, [&] { m.f64.rot.alloc(9 * m.n); });
     pdl_launch(k_rotations<double>, grid, 128, 0, s, m.n, (const int32_t*)m.d_nbr_ptr.p,
                (const int32_t*)m.d_nbr_idx.p, x, (const double*)m.d_Xrest.p, m.f64.rot.p);
   }

@@ -1412,6 +1412,10 @@ cc_status cc_build_learned_subspace(cc_mesh* m, cc_mlp* net, double tau, double*
     CCG_CUDA(cudaStreamSynchronize(s));
     out.ms_fallback = ms_since(t0);
 
+    t0 = std::chrono::steady_clock::now();
+    ensure_coupling_lists(*m, true);
+    out.ms_supports += ms_since(t0);
+
     out.n_free = nf;
     out.n_fallback = (int64_t)fall.size();
     out.rho_max = rmax;
