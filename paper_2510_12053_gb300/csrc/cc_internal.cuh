@@ -23,10 +23,13 @@ struct Fail {
   cc_status st;
 };
 
+// A failed call's error is also the runtime's last error: it is taken back, or
+// the next launch check on this thread would report it again.
 #define CCG_CUDA(call)                                                                     \
   do {                                                                                     \
     cudaError_t e_ = (call);                                                               \
     if (e_ != cudaSuccess) {                                                               \
+      cudaGetLastError();                                                                  \
       ::ccg::set_error(std::string(#call) + ": " + cudaGetErrorString(e_));               \
       throw ::ccg::Fail{e_ == cudaErrorMemoryAllocation ? CC_ERR_OOM : CC_ERR_CUDA};      \
     }                                                                                      \

@@ -417,7 +417,6 @@ static void build_pair_lists(Mesh& m) {
     m.d_sup_row.release();
     m.d_pairs.release();
     if (f.st != CC_ERR_OOM) throw;
-    cudaGetLastError();
     clear_error();
   }
 }
@@ -495,7 +494,6 @@ void ensure_coupling_lists(Mesh& m, bool mixed) {
 
 bool drop_pair_lists(Mesh& m) {
   if (!m.pairs_ok) return false;
-  cudaGetLastError();
   clear_error();
   drop_graph(m);  // its nodes read the lists
   m.pairs_ok = false;

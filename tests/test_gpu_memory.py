@@ -106,3 +106,22 @@ def test_solver_state_takes_the_place_of_the_pair_lists(body):
         torch.cuda.empty_cache()
     m.close()
     assert np.abs(got - want).max() <= 1e-4 * np.abs(want).max()
+
+
+def test_a_call_after_one_that_ran_out_of_memory_works(body):
+    sc, sizes, want = body
+    m, x = _mesh(sc)
+    hold = _leave(sizes["bases"] / 2)
+    try:
+        with pytest.raises(cc.CCError) as e:
+            m.build_subspace(2)
+        assert e.value.status == cc.ERR_OOM
+    finally:
+        del hold
+        torch.cuda.empty_cache()
+    with pytest.raises(cc.CCError):  # no subspace, so no sweep that reads one
+        m.sweep(x, precision="mixed")
+    m.build_subspace(2)
+    m.sweep(x, precision="mixed")
+    m.close()
+    assert np.abs(cc.from_soa(x) - sc.x0 - want).max() <= 1e-4 * np.abs(want).max()
