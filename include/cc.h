@@ -422,8 +422,10 @@ cc_status cc_solve_concurrent(int32_t count, cc_mesh* const* meshes, double* con
  * (cc_set_sweep_variant), threads per vertex of the coupling kernel (32 = one
  * warp per vertex, 64, 128, 256), then, unless one warp won, threads per
  * block row of the coupling kernel (1, 2, 4, 8), then block rows per CTA of
- * the row gather (2, 4, 8 warps); it keeps the fastest of each for this
- * mesh.  x_dev is not modified (the sweeps run on a private copy).  Requires
+ * the row gather (2, 4, 8 warps); it keeps the fastest of each for this mesh,
+ * and the row build for this precision only.  Rows from the positions are not tried in the mixed path of a dynamic
+ * mesh unless the caller has switched them on.
+ * x_dev is not modified (the sweeps run on a private copy).  Requires
  * cc_color and a subspace.  Results with different configurations agree to
  * the working precision's rounding (the coupling kernel's partial sums are
  * grouped differently). */
@@ -472,7 +474,7 @@ cc_status cc_set_launch_shape(cc_mesh* mesh, int32_t couple_threads, int32_t gat
  * rounding (v = dx / h shows it), and for the float64 path of a mesh with a
  * vertex of more than about 55 tets (the gather is faster there);
  * fused_condense 0 (measured fastest).
- * cc_autotune tries every applicable combination.  The fused and separate
+ * cc_autotune tries the applicable combinations.  The fused and separate
  * condensations give identical results; the two row builds agree within the
  * rounding of the path's precision. */
 cc_status cc_set_sweep_variant(cc_mesh* mesh, int32_t rows_from_positions, int32_t fused_condense);

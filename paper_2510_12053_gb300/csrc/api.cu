@@ -1131,6 +1131,7 @@ cc_status cc_autotune(cc_mesh* m, const double* x, const double* xt, cc_precisio
     CCG_CUDA(cudaEventCreate(&e1));
     const bool prof = m->prof.on;
     m->prof.on = false;
+    const int ct0 = m->tune_couple_threads;
     auto time_sweeps = [&]() -> double {
       CCG_CUDA(cudaMemcpyAsync(tmp.p, x, 3 * m->n * sizeof(double), cudaMemcpyDeviceToDevice, s));
       activate_all(*m);
@@ -1153,27 +1154,28 @@ cc_status cc_autotune(cc_mesh* m, const double* x, const double* xt, cc_precisio
       return ms / sweeps;
     };
     try {
-      // sweep variant first, at the current launch shapes
+      // sweep variant first, at the current launch shapes.  A dynamic mesh's mixed
+      // rows keep their float32 rounding unless the caller has switched it, so
+      // timing does not.
+      const bool mixed = p == CC_PREC_MIXED;
       {
-        const int rb0 = m->rows_build;
-        const bool fc0 = m->fused_condense;
         int best_v = -1;
         for (int v = 0; v < 4; ++v) {
           out->variant_ms[v] = 0.0;
-          m->rows_build = v >> 1;
+          m->rows_tuned[mixed] = v >> 1;
           m->fused_condense = (v & 1) != 0;
-          if (m->rows_build && !rows_from_positions(*m, p == CC_PREC_MIXED)) continue;  // not applicable
+          if ((v >> 1) != 0 && (!m->rows_ok || (mixed_dynamic(*m, mixed) && m->rows_build != 1))) continue;
           ensure_state(*m, p);
           drop_graph(*m);
           out->variant_ms[v] = time_sweeps();
           if (best_v < 0 || out->variant_ms[v] < out->variant_ms[best_v]) best_v = v;
         }
-        m->rows_build = best_v >= 0 ? best_v >> 1 : rb0;
-        m->fused_condense = best_v >= 0 ? (best_v & 1) != 0 : fc0;
+        m->rows_tuned[mixed] = best_v >> 1;
+        if (rows_from_positions(*m, mixed) == rows_by_switch(*m, mixed)) m->rows_tuned[mixed] = -1;
+        m->fused_condense = (best_v & 1) != 0;
         ensure_state(*m, p);
       }
       const int ct[4] = {32, 64, 128, 256}, gw[3] = {2, 4, 8};
-      const int ct0 = m->tune_couple_threads;
       for (int k = 0; k < 4; ++k) {
         m->tune_couple_threads = ct[k];
         try {
@@ -1253,7 +1255,10 @@ cc_status cc_set_sweep_variant(cc_mesh* m, int32_t rows_from_positions, int32_t 
     CCG_CHECK(m, CC_ERR_INVALID_ARG, "mesh is NULL");
     CCG_CHECK(rows_from_positions >= -1 && rows_from_positions <= 1 && fused_condense >= -1 && fused_condense <= 1,
               CC_ERR_INVALID_ARG, "variant switches are 1 (on), 0 (off) or -1 (keep)");
-    if (rows_from_positions >= 0) m->rows_build = rows_from_positions;
+    if (rows_from_positions >= 0) {
+      m->rows_build = rows_from_positions;
+      m->rows_tuned[0] = m->rows_tuned[1] = -1;
+    }
     if (fused_condense >= 0) m->fused_condense = fused_condense != 0;
     drop_graph(*m);
     // what the chosen row build needs (the per-tet store or the per-tet sigma)

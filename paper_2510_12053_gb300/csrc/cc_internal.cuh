@@ -176,7 +176,8 @@ struct Mesh {
   int tune_couple_row_lanes = 4;  // threads per block row in the coupling kernel (1, 2, 4, 8)
   int tune_gather_wpb = 4;        // warps (rows) per block in the row gather
   bool fused_condense = false;    // the coupling kernel's last CTA of every 32 vertices condenses them
-  int rows_build = -1;            // rows formed from the positions (kernels_rows.cu): 1, 0, -1 by rows_from_positions
+  int rows_build = -1;            // rows formed from the positions (kernels_rows.cu): the caller's switch, 1, 0, -1 unset
+  int rows_tuned[2] = {-1, -1};   // cc_autotune's choice for the float64 and the mixed sweeps, -1 none
   int64_t n = 0, T = 0, n_free = 0, nnzb = 0;
   int32_t max_valence = 0;
   double E = 0, nu = 0, rho = 0, mu = 0, lam_hat = 0, h = 0;
@@ -365,14 +366,20 @@ inline bool mixed_dynamic(const Mesh& m, bool mixed) { return mixed && m.h > 0.0
 
 inline bool couples_from_pairs(const Mesh& m, bool mixed) { return !mixed_dynamic(m, mixed); }
 
-inline bool rows_from_positions(const Mesh& m, bool mixed) {
+// Row build of a precision's sweeps: tuned, else switched, else the default.
+inline bool rows_by_switch(const Mesh& m, bool mixed) {
   const bool by_default = mixed ? !mixed_dynamic(m, mixed) : m.rows64_fast;
   return m.rows_ok && (m.rows_build < 0 ? by_default : m.rows_build != 0);
 }
 
-// The float64 Hessian that bases are built from: a dynamic mesh's keeps the
-// store with its float32 path (whose float32 copies of the bases it rounds).
-inline bool bases_from_positions(const Mesh& m) { return rows_from_positions(m, m.h > 0.0); }
+inline bool rows_from_positions(const Mesh& m, bool mixed) {
+  return m.rows_tuned[mixed] < 0 ? rows_by_switch(m, mixed) : m.rows_ok && m.rows_tuned[mixed] != 0;
+}
+
+// The float64 Hessian that bases are built from (tuning a sweep leaves it): a
+// dynamic mesh's keeps the store with its float32 path (whose float32 copies of
+// the bases it rounds).
+inline bool bases_from_positions(const Mesh& m) { return rows_by_switch(m, m.h > 0.0); }
 
 template <typename... KArgs, typename... Args>
 void pdl_launch(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args&&... args) {
