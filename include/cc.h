@@ -424,7 +424,9 @@ cc_status cc_solve_concurrent(int32_t count, cc_mesh* const* meshes, double* con
  * block row of the coupling kernel (1, 2, 4, 8), then block rows per CTA of
  * the row gather (2, 4, 8 warps); it keeps the fastest of each for this mesh,
  * and the row build for this precision only.  Rows from the positions are not tried in the mixed path of a dynamic
- * mesh unless the caller has switched them on.
+ * mesh unless the caller has switched them on; a variant whose buffers find no
+ * memory is left out, and buffers that the choice does not read are given back.
+ * A call that fails leaves every setting as it was.
  * x_dev is not modified (the sweeps run on a private copy).  Requires
  * cc_color and a subspace.  Results with different configurations agree to
  * the working precision's rounding (the coupling kernel's partial sums are
@@ -469,6 +471,7 @@ cc_status cc_set_launch_shape(cc_mesh* mesh, int32_t couple_threads, int32_t gat
  *                        lane); 0: a separate condensation launch.  The
  *                        one-warp coupling shape always launches it apart.
  * 1 sets, 0 clears, -1 keeps a switch; anything else is CC_ERR_INVALID_ARG.
+ * CC_ERR_OOM (the rows' buffers find no memory) changes nothing.
  * Defaults: rows_from_positions 1 (measured fastest), but 0 for the mixed
  * path of a dynamic mesh (h > 0), whose steps keep the gather's float32
  * rounding (v = dx / h shows it), and for the float64 path of a mesh with a

@@ -105,6 +105,18 @@ static void alloc_state(Mesh& m, cc_precision p) {
   }
 }
 
+// Gives back the per-tet stores that the row builds in use do not read.
+static void release_unused_store(Mesh& m) {
+  if (rows_from_positions(m, true)) {
+    m.mx.gcon.release();
+    m.mx.hten.release();
+  }
+  if (rows_from_positions(m, false) && bases_from_positions(m)) {
+    m.f64.gcon.release();
+    m.f64.hten.release();
+  }
+}
+
 bool state_allocated(const Mesh& m, cc_precision p) {
   return p == CC_PREC_FP64 ? m.f64.cpl.p != nullptr : m.mx.xt_lo.p != nullptr;
 }
@@ -1131,7 +1143,9 @@ cc_status cc_autotune(cc_mesh* m, const double* x, const double* xt, cc_precisio
     CCG_CUDA(cudaEventCreate(&e1));
     const bool prof = m->prof.on;
     m->prof.on = false;
-    const int ct0 = m->tune_couple_threads;
+    const int tuned0 = m->rows_tuned[p == CC_PREC_MIXED], ct0 = m->tune_couple_threads, rl0 = m->tune_couple_row_lanes,
+              gw0 = m->tune_gather_wpb;
+    const bool fused0 = m->fused_condense;
     auto time_sweeps = [&]() -> double {
       CCG_CUDA(cudaMemcpyAsync(tmp.p, x, 3 * m->n * sizeof(double), cudaMemcpyDeviceToDevice, s));
       activate_all(*m);
@@ -1156,7 +1170,7 @@ cc_status cc_autotune(cc_mesh* m, const double* x, const double* xt, cc_precisio
     try {
       // sweep variant first, at the current launch shapes.  A dynamic mesh's mixed
       // rows keep their float32 rounding unless the caller has switched it, so
-      // timing does not.
+      // timing does not; a variant without memory for its buffers is left out.
       const bool mixed = p == CC_PREC_MIXED;
       {
         int best_v = -1;
@@ -1165,15 +1179,23 @@ cc_status cc_autotune(cc_mesh* m, const double* x, const double* xt, cc_precisio
           m->rows_tuned[mixed] = v >> 1;
           m->fused_condense = (v & 1) != 0;
           if ((v >> 1) != 0 && (!m->rows_ok || (mixed_dynamic(*m, mixed) && m->rows_build != 1))) continue;
-          ensure_state(*m, p);
           drop_graph(*m);
+          try {
+            alloc_state(*m, p);
+          } catch (const Fail& f) {
+            if (f.st != CC_ERR_OOM) throw;
+            clear_error();
+            continue;
+          }
           out->variant_ms[v] = time_sweeps();
           if (best_v < 0 || out->variant_ms[v] < out->variant_ms[best_v]) best_v = v;
         }
+        CCG_CHECK(best_v >= 0, CC_ERR_OOM, "no sweep variant fits the device memory");
         m->rows_tuned[mixed] = best_v >> 1;
         if (rows_from_positions(*m, mixed) == rows_by_switch(*m, mixed)) m->rows_tuned[mixed] = -1;
         m->fused_condense = (best_v & 1) != 0;
         ensure_state(*m, p);
+        release_unused_store(*m);
       }
       const int ct[4] = {32, 64, 128, 256}, gw[3] = {2, 4, 8};
       for (int k = 0; k < 4; ++k) {
@@ -1212,7 +1234,14 @@ cc_status cc_autotune(cc_mesh* m, const double* x, const double* xt, cc_precisio
       for (int k = 1; k < 3; ++k)
         if (out->gather_ms[k] < out->gather_ms[best]) best = k;
       m->tune_gather_wpb = gw[best];
-    } catch (...) {
+    } catch (...) {  // everything as it was
+      m->rows_tuned[p == CC_PREC_MIXED] = tuned0;
+      m->fused_condense = fused0;
+      m->tune_couple_threads = ct0;
+      m->tune_couple_row_lanes = rl0;
+      m->tune_gather_wpb = gw0;
+      drop_graph(*m);
+      release_unused_store(*m);
       m->prof.on = prof;
       cudaEventDestroy(e0);
       cudaEventDestroy(e1);
@@ -1255,15 +1284,23 @@ cc_status cc_set_sweep_variant(cc_mesh* m, int32_t rows_from_positions, int32_t 
     CCG_CHECK(m, CC_ERR_INVALID_ARG, "mesh is NULL");
     CCG_CHECK(rows_from_positions >= -1 && rows_from_positions <= 1 && fused_condense >= -1 && fused_condense <= 1,
               CC_ERR_INVALID_ARG, "variant switches are 1 (on), 0 (off) or -1 (keep)");
+    const int build0 = m->rows_build, tuned0[2] = {m->rows_tuned[0], m->rows_tuned[1]};
+    drop_graph(*m);
     if (rows_from_positions >= 0) {
       m->rows_build = rows_from_positions;
       m->rows_tuned[0] = m->rows_tuned[1] = -1;
     }
+    try {
+      // what the chosen row build needs (the per-tet store or the per-tet sigma)
+      if (state_allocated(*m, CC_PREC_MIXED)) ensure_state(*m, CC_PREC_MIXED);
+      if (state_allocated(*m, CC_PREC_FP64)) ensure_state(*m, CC_PREC_FP64);
+    } catch (...) {
+      m->rows_build = build0;
+      m->rows_tuned[0] = tuned0[0];
+      m->rows_tuned[1] = tuned0[1];
+      throw;
+    }
     if (fused_condense >= 0) m->fused_condense = fused_condense != 0;
-    drop_graph(*m);
-    // what the chosen row build needs (the per-tet store or the per-tet sigma)
-    if (state_allocated(*m, CC_PREC_MIXED)) ensure_state(*m, CC_PREC_MIXED);
-    if (state_allocated(*m, CC_PREC_FP64)) ensure_state(*m, CC_PREC_FP64);
   })
 }
 

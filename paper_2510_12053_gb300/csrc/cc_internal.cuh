@@ -413,14 +413,17 @@ void reset_coupling_lists(Mesh& m);
 // false when there are none.
 bool drop_pair_lists(Mesh& m);
 // Runs f, which allocates.  The pair lists are only the faster way: where f
-// finds no memory beside them it runs again without them.
+// finds no memory beside them it runs again without them.  If that fails too,
+// the next sweep may make them again.
 template <typename F>
 void with_room(Mesh& m, F&& f) {
   try {
     f();
   } catch (const Fail& e) {
     if (e.st != CC_ERR_OOM || !drop_pair_lists(m)) throw;
+    m.pairs_tried = false;
     f();
+    m.pairs_tried = true;
   }
 }
 // host worker threads for setup passes, and a parallel loop over vertex ranges

@@ -488,7 +488,16 @@ void reset_coupling_lists(Mesh& m) {
 
 void ensure_coupling_lists(Mesh& m, bool mixed) {
   const bool pairs = couples_from_pairs(m, mixed);
-  if (pairs && !m.pairs_tried) build_pair_lists(m);
+  if (pairs && !m.pairs_tried) {
+    build_pair_lists(m);
+    if (m.pairs_ok && m.smap_ok) drop_graph(m);  // captured over the slot maps
+    if (m.pairs_ok && couples_from_pairs(m, true)) {  // no sweep of this mesh reads them now
+      m.smap_ok = false;
+      m.d_smap_ptr.release();
+      m.d_smap8.release();
+      m.d_smap16.release();
+    }
+  }
   if (!(pairs && m.pairs_ok) && !m.smap_ok) build_slot_maps(m);
 }
 
