@@ -421,9 +421,11 @@ cc_status cc_solve_concurrent(int32_t count, cc_mesh* const* meshes, double* con
  * one parameter at a time in this order: the sweep variant
  * (cc_set_sweep_variant), threads per vertex of the coupling kernel (32 = one
  * warp per vertex, 64, 128, 256), then, unless one warp won, threads per
- * block row of the coupling kernel (1, 2, 4, 8), then block rows per CTA of
- * the row gather (2, 4, 8 warps); it keeps the fastest of each for this mesh,
- * and the row build for this precision only.  Rows from the positions are not tried in the mixed path of a dynamic
+ * block row of the coupling kernel (1, 2, 4, 8; where that kernel has no such
+ * threads, see cc_set_launch_shape, the setting stays and its four times are the
+ * chosen shape's), then block rows per CTA of the row gather (2, 4, 8 warps); it
+ * keeps the fastest of each for this mesh, and the row build for this precision
+ * only.  Rows from the positions are not tried in the mixed path of a dynamic
  * mesh unless the caller has switched them on; a variant whose buffers find no
  * memory is left out, and buffers that the choice does not read are given back.
  * A call that fails leaves every setting as it was.

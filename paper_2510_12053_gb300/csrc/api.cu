@@ -1217,7 +1217,10 @@ cc_status cc_autotune(cc_mesh* m, const double* x, const double* xt, cc_precisio
       const int rl[4] = {1, 2, 4, 8};
       int best_rl = -1;
       for (int k = 0; k < 4; ++k) out->row_lanes_ms[k] = 0.0;
-      if (m->tune_couple_threads != 32) {  // the one-warp kernel splits blocks, not rows
+      if (m->pairs_ok && couples_from_pairs(*m, mixed)) {  // its kernels have no row lanes: one time for all four
+        if (m->tune_couple_threads != 32)
+          for (int k = 0; k < 4; ++k) out->row_lanes_ms[k] = out->couple_ms[best];
+      } else if (m->tune_couple_threads != 32) {  // the one-warp kernel splits blocks, not rows
         const int keep = m->tune_couple_row_lanes;
         for (int k = 0; k < 4; ++k) {
           m->tune_couple_row_lanes = rl[k];

@@ -57,6 +57,18 @@ def test_a_switched_dynamic_mesh_is_tuned_over_both_row_builds():
     m.close()
 
 
+def test_row_lanes_are_not_chosen_for_kernels_without_them():
+    sc = meshgen.stretch_box(5, 4, 6, E=1e5, nu=0.3, factor=1.05, jitter_amount=0.05, seed=8)
+    m = cc.Mesh.from_scene(sc)
+    m.color()
+    m.build_subspace(2)
+    m.set_launch_shape(couple_row_lanes=2)
+    for precision in ("mixed", "fp64"):
+        tune = m.autotune(cc.to_soa(sc.x0), precision=precision, sweeps=2)
+        assert tune["couple_row_lanes"] == 2 and len(set(tune["row_lanes_ms"])) == 1
+    m.close()
+
+
 def _free():
     torch.cuda.synchronize()
     return torch.cuda.mem_get_info()[0]
