@@ -483,35 +483,24 @@ def local_solve_flops(mesh):
     return out
 
 
-def gather_bytes_per_refresh(scene):
-    """Algorithmic bytes of one row-gather launch (all free rows): per row the
-    stored blocks it sums (per incident tet its 24-byte diagonal block and a
-    36-byte block per other corner with a vertex id above the row's), its
-    24-byte float-float gradient entries, its upper blocks written and its
-    gradient written."""
-    tets = np.asarray(scene.tets, dtype=np.int64)
-    free = scene.pinned == 0
-    n = scene.n
-    ge = tets[:, None, :] >= tets[:, :, None]          # [T, v, w]: vid[w] >= vid[v]
-    src = np.zeros(n)
-    np.add.at(src, tets.ravel(), ge.sum(axis=2).ravel())
-    val = np.bincount(tets.ravel(), minlength=n)
-    nup = np.zeros(n)
-    pairs = set()
-    for a in range(4):
-        for c in range(4):
-            if a != c:
-                pairs.update(zip(tets[:, a].tolist(), tets[:, c].tolist()))
-    for (j, l) in pairs:
-        if l > j:
-            nup[j] += 1
-    nup += 1
-    per = (src - val) * 36 + val * 24 + val * 24 + nup * 36 + 24
-    return float(per[free].sum())
+def rows_bytes_per_refresh(mesh, scene):
+    """Algorithmic bytes of one launch that forms all free rows from the
+    positions (mixed path): per row its record and diagonal constant (36 B) and
+    own position (32 B), per 1-ring neighbour its id, weight and position
+    (44 B), per incident tet its id, ring slots and sigma record (24 B), per
+    off-diagonal upper block its source codes (16 B); written, 48 B per upper
+    block, the gradient (24 B) and the (H_jj, g_j) record (48 B)."""
+    nbp, nbi = mesh.export("nbr_ptr"), mesh.export("nbr_idx")
+    ring = np.diff(nbp)
+    owner = np.repeat(np.arange(scene.n), ring)
+    nup = np.bincount(owner[nbi > owner], minlength=scene.n) + 1
+    val = np.bincount(np.asarray(scene.tets, dtype=np.int64).ravel(), minlength=scene.n)
+    per = 68 + ring * 44 + val * 24 + (nup - 1) * 16 + nup * 48 + 72
+    return float(per[scene.pinned == 0].sum())
 
 
-# ids, slots, D_m^-1, V w, positions; gradient + 10 blocks (4 diagonal ones as 6 values, 6 others as 9)
-TET_BYTES = 16 + 16 + 72 + 12 + 4 * 32 + 4 * 24 + 4 * (4 * 6 + 6 * 9)
+# k_tet_sigma: list entry, vertex ids, coefficients, four positions; record written
+TET_BYTES = 4 + 16 + 16 + 4 * 32 + 16
 
 
 def run_batch(args, stream, dev):
@@ -709,17 +698,7 @@ def run_large(args, stream, dev):
     m.profile_enable(False)
     ms = ev0.elapsed_time(ev1)
     ncol = int(m.info().num_colors)
-    # algorithmic bytes (vectorised forms of the per-unit figures used for the cube)
-    tets = np.asarray(sc.tets, dtype=np.int64)
-    ge = tets[:, None, :] >= tets[:, :, None]
-    src = np.zeros(sc.n)
-    np.add.at(src, tets.ravel(), ge.sum(axis=2).ravel())
-    val = np.bincount(tets.ravel(), minlength=sc.n)
-    nbp, nbi = m.export("nbr_ptr"), m.export("nbr_idx")
-    owner = np.repeat(np.arange(sc.n), np.diff(nbp))
-    nup = np.bincount(owner[nbi > owner], minlength=sc.n) + 1
-    free = sc.pinned == 0
-    gather_bytes = float(((src - val) * 36 + val * 24 + val * 24 + nup * 36 + 24)[free].sum())
+    gather_bytes = rows_bytes_per_refresh(m, sc)
     free_corners = int((sc.pinned[sc.tets] == 0).sum())
     active_tets = int((sc.pinned[sc.tets] == 0).any(axis=1).sum())
     tet_refreshes = r.iterations * free_corners + active_tets
@@ -995,7 +974,7 @@ def run_learned(args, stream, dev):
     return out
 
 
-SWEEP_KERNELS = ("k_tet_grad_mixed", "k_row_gather", "k_couple", "k_condense")
+SWEEP_KERNELS = ("k_tet_sigma", "k_rows_mixed", "k_couple_pairs", "k_condense")
 
 
 def sweep_ncu_traffic(ncol):
@@ -1011,8 +990,8 @@ def per_class_rooflines(cls, meshes, scs, sweeps, tet_refreshes, row_gathers, fl
     ls = cls["local_solve"]
     if ls["ms"] > 0:
         ach = flops_per_sweep * sweeps / (ls["ms"] / 1e3) / 1e12
-        tr = [ncu_traffic("k_couple"), ncu_traffic("k_condense")]
-        roof["local_solve"] = {"kernel": "k_couple + k_condense (coupling products + batched Schur solve)",
+        tr = [ncu_traffic("k_couple_pairs"), ncu_traffic("k_condense")]
+        roof["local_solve"] = {"kernel": "k_couple_pairs + k_condense (coupling products + batched Schur solve)",
                                "bound": "alu", "achieved": ach, "peak": FP32_PEAK_TFLOPS, "unit": "TFLOP/s",
                                "frac": ach / FP32_PEAK_TFLOPS,
                                "traffic": (tr[0] + tr[1]) if None not in tr else None,
@@ -1021,20 +1000,20 @@ def per_class_rooflines(cls, meshes, scs, sweeps, tet_refreshes, row_gathers, fl
                                "avg_launch_ms": ls["ms"] / max(ls["launches"] // 2, 1)}
     ga = cls["gather"]
     if ga["ms"] > 0:
-        gb = gather_bytes_per_refresh(scs[0])
+        gb = rows_bytes_per_refresh(meshes[0], scs[0])
         ach = gb * row_gathers / (ga["ms"] / 1e3) / 1e9
-        roof["gather"] = {"kernel": "k_row_gather (gradient + upper block rows of every free vertex)",
+        roof["gather"] = {"kernel": "k_rows_mixed (gradient + upper block rows of every free vertex from the positions)",
                           "bound": "hbm", "achieved": ach, "peak": hbm, "unit": "GB/s", "frac": ach / hbm,
-                          "traffic": ncu_traffic("k_row_gather"), "peak_source": peak_src,
-                          "algorithmic": f"{gb / 1e6:.1f} MB per launch (counts the per-tet Hessian store, "
-                                         f"which the sweep roofline treats as overhead)",
+                          "traffic": ncu_traffic("k_rows_mixed"), "peak_source": peak_src,
+                          "algorithmic": f"{gb / 1e6:.1f} MB per launch (counts the block rows, which the sweep "
+                                         f"roofline treats as overhead)",
                           "avg_launch_ms": ga["ms"] / max(ga["launches"], 1)}
     te = cls["tet_eval"]
     if te["ms"] > 0:
         ach = TET_BYTES * tet_refreshes / (te["ms"] / 1e3) / 1e9
-        roof["tet_eval"] = {"kernel": "k_tet_grad_mixed (float-float gradient + float32 Hessian blocks per tet)",
+        roof["tet_eval"] = {"kernel": "k_tet_sigma (one float-float coefficient per tet)",
                             "bound": "hbm", "achieved": ach, "peak": hbm, "unit": "GB/s", "frac": ach / hbm,
-                            "traffic": ncu_traffic("k_tet_grad_mixed"), "peak_source": peak_src,
+                            "traffic": ncu_traffic("k_tet_sigma"), "peak_source": peak_src,
                             "algorithmic": f"{TET_BYTES} B per refreshed tet",
                             "avg_launch_ms": te["ms"] / max(te["launches"], 1)}
     return roof
