@@ -105,11 +105,15 @@ static void alloc_state(Mesh& m, cc_precision p) {
   }
 }
 
-// Gives back the per-tet stores that the row builds in use do not read.
+// Gives back what the row builds in use do not read: a per-tet store, or the
+// records of rows formed from the positions.
 static void release_unused_store(Mesh& m) {
   if (rows_from_positions(m, true)) {
     m.mx.gcon.release();
     m.mx.hten.release();
+  } else {
+    m.mx.diag_g.release();
+    m.mx.rec.release();
   }
   if (rows_from_positions(m, false) && bases_from_positions(m)) {
     m.f64.gcon.release();

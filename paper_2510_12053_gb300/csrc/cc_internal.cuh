@@ -347,10 +347,6 @@ constexpr size_t kRowsSmemMax = 200 * 1024;
 // 240 (32^3 cells: 66 / 31 us at 24, 148 / 112 at 240).
 constexpr size_t kRows64FastSmem = 40 * 1024;
 
-// Stable Neo-Hookean block rows are formed from the positions instead of a
-// per-tet Hessian store (kernels_rows.cu); Fixed Corotational keeps the store
-// (its blocks need the polar rotation, too costly to form four times per tet),
-// and so do meshes whose rows do not fit that kernel.
 // The coupling kernel condenses its vertices itself (one launch per colour
 // for the local solves) unless switched off or with the one-warp coupling kernel.
 inline bool fused_local_solve(const Mesh& m, cc_update upd) {
@@ -360,12 +356,19 @@ inline bool fused_local_solve(const Mesh& m, cc_update upd) {
 // A dynamic mesh's float32 path keeps the store, and the slot-map coupling
 // kernel, unless switched on: a step returns v = (x_new - x_old) / h, which
 // shows the float32 rounding of the updates at full relative size (1e-7),
-// where positions show it four to five digits lower; so its sums keep the order
-// they have always had, and a step its bits.
+// where positions show it four to five digits lower.  So its float32 sums keep
+// the order they have always had, and a step its bits for given bases (those of
+// patches up to kPmMaxN unknowns come from another factorisation by now: 1e-13
+// off, and now and then a float32 copy that rounds the other way).  Whether the
+// other kernels' v is further from float64 has not been measured.
 inline bool mixed_dynamic(const Mesh& m, bool mixed) { return mixed && m.h > 0.0; }
 
 inline bool couples_from_pairs(const Mesh& m, bool mixed) { return !mixed_dynamic(m, mixed); }
 
+// Stable Neo-Hookean block rows are formed from the positions instead of a
+// per-tet Hessian store (kernels_rows.cu); Fixed Corotational keeps the store
+// (its blocks need the polar rotation, too costly to form four times per tet),
+// and so do meshes whose rows do not fit that kernel.
 // Row build of a precision's sweeps: tuned, else switched, else the default.
 inline bool rows_by_switch(const Mesh& m, bool mixed) {
   const bool by_default = mixed ? !mixed_dynamic(m, mixed) : m.rows64_fast;

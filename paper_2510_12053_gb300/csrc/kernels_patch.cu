@@ -20,8 +20,9 @@
 // use the inverted diagonal tiles: two barriers per 16 unknowns.  The residual
 // takes a thread per (row block, right-hand side) over a list of the row's
 // blocks inside the patch, found once.
-// What bounds it: the float64 residual (about 6 000 block products a patch
-// and iteration) and the shared-memory reads of the tile updates together.
+// What bounds it: the float64 residual (an interior 2-ring of a Kuhn grid lists
+// 644 blocks: 1 932 products with one right-hand side, 17 400 fused operations
+// an iteration) and the shared-memory reads of the tile updates together.
 // A column-by-column factorisation in packed storage (two barriers and one
 // rank-one update per unknown), one thread per row in the residual with its
 // neighbours searched again in every iteration, made a solve of the 16^3 cube
@@ -37,7 +38,7 @@ constexpr int kPmThreads = 256;
 constexpr int kPmWarps = kPmThreads / 32;
 constexpr int kPmTiles = kPmMaxN / 16;
 constexpr int kPmTileFloats = 256 * kPmTiles * (kPmTiles + 1) / 2;
-constexpr int kPmMaxBlocks = 1280;  // listed blocks of a patch (an interior 2-ring of a Kuhn grid: 650)
+constexpr int kPmMaxBlocks = 1280;  // listed blocks of a patch (an interior 2-ring of a Kuhn grid: 644)
 static_assert(kPmMaxN % 16 == 0 && kPmMaxN <= kPmThreads && kPmMaxN / 3 <= 255, "patch kernel sizes");
 
 struct PatchSmem {

@@ -146,7 +146,8 @@ __host__ __device__ inline size_t rows_mixed_smem(int max_val, int max_ring) {
 //      operations) costs no more than staging seven vectors per (row, tet) in
 //      step 2, and keeps a row at 0.8 KB of shared memory instead of 2.7 KB
 //      (staged: 30.9 us against 24.0 on the 32^3 cube, 16 warps an SM
-//      against 24).  Instruction issue bounds it (13.3 M warp instructions).
+//      against 24).  Instruction issue bounds it (13.3 M warp instructions);
+//      80 registers, 8 bytes a thread spilled.
 __global__ void __launch_bounds__(256, 3) k_rows_mixed(
     const int4* __restrict__ hdr, int64_t nrows, const int32_t* __restrict__ nbr_idx,
     const float2* __restrict__ ring_m, const float* __restrict__ row_diag, const int32_t* __restrict__ vt_tet,

@@ -10,8 +10,8 @@
 // and x_i += dx_i (the subspace part U dalpha is discarded, Sec. 3.1).
 // H is stored as its upper 3x3 blocks (l >= j, diagonal first, each block
 // padded to 3 x 4 for 128-bit loads), so each unordered pair of the support
-// is read once.  The CTA stages U_i in shared memory; a precomputed slot map
-// gives, for every block it reads, the support slot of the block's column.
+// is read once.  The CTA stages U_i in shared memory; a precomputed pair list
+// (or slot map) gives, for every block it reads, the support slot of the block's column.
 // Same-coloured vertices share no tet, and this kernel reads only g, H and U,
 // so writing x in place is race-free for both schedules.
 #include <vector>
@@ -914,7 +914,9 @@ __device__ __forceinline__ void reduce18(const HT* M, const HT* A, const HT* b, 
 // loads after the vertex number, and no thread walks blocks outside the support.
 // Bound by L1 wavefronts (72% of peak) and load latency together: 39 us a colour
 // of the 32^3 cube (8 440 vertices) cold, 50 k wavefronts an SM; the slot-map
-// kernel above took 46 us.  64 registers (16 CTAs of 64 threads an SM).
+// kernel above took 46 us.  64 registers (16 CTAs of 64 threads an SM), at which
+// the CC update spills a little: 20 bytes stored and 32 loaded a thread with two
+// to eight warps, 4 and 4 with one warp and two shares.
 // kShares: the loops' work is dealt to kShares x kThreads threads, and the CTA
 // takes the shares one after the other; each share's sums are reduced by
 // themselves, so one warp with two shares gives the bits of two warps.
